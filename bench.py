@@ -745,18 +745,16 @@ def bench_serve(cs, torch, factors=(0.5, 0.9, 1.5), count=120, seed=2026):
 
 
 def ch_fp64_ops_per_point(chunks: int, m: int, fp32_storage: bool = False) -> float:
-    """FP64-pipe operations per grid point of one ADI step as the kernels perform them (ncu's
-    DFMA + DADD + DMUL counts of the 4096^2 FP64 step: 5.45 + 5 + 5 + 5 + 6 = 26.4 at 16 chunks
-    of 256).  The right-hand side, per CTA of 64 x 32 points: Cbar = 2 C^n - C^{n-1} on the 68 x 36
-    halo-2 tile (one FMA; FP32 storage forms it in FP32), Z's one digit-combination FMA on the
-    66 x 34 halo-1 tile (the cubic term joins the integer digit sum), then per point the second
-    combination, C^n - C^{n-1} and the final FMA, and one multiply per thread for the combination's
-    constant.  Each sweep: local LU 4 FMAs and 1 multiply, the spike correction 4 FMAs and the
-    chunk-end system 16 chunks / m.  The update: one add (Cbar comes from the right-hand side kernel
-    through the C^{n+1} buffer; FP32 storage narrows on the integer pipe)."""
+    """FP64-pipe operations per grid point of one ADI step.  The right-hand side, per CTA of
+    64 x 32 points: Cbar = 2 C^n - C^{n-1} on the 68 x 36 halo-2 tile (one FMA; FP32 storage forms it
+    in FP32), Z's one digit-combination FMA on the 66 x 34 halo-1 tile (the cubic term joins the
+    integer digit sum), then per point the second combination, C^n - C^{n-1} and the final FMA, and one
+    multiply per thread for the combination's constant.  The line solves run in fixed point; per chunk
+    and sweep the scan over a line's chunks (4 FMAs per level, forward and backward, and 4 between
+    them) and 8 conversions are FP64.  The update: one add."""
     tile = 64 * 32
     rhs = (0 if fp32_storage else 68 * 36 / tile) + 66 * 34 / tile + 3 + 256 / tile
-    per_sweep = 5 + 4 + 16.0 * chunks / m
+    per_sweep = (8 * int(np.ceil(np.log2(max(chunks, 2)))) + 12) / m
     return rhs + 2 * per_sweep + 1
 
 

@@ -352,18 +352,18 @@ int cs_ch_config(cs_plan_t plan, int32_t* chunks, int32_t* chunk_len);
  * Steps 1, 4 and 6 are the caller's communication (paper_1902_09931_gb300.distributed does them
  * with torch.distributed); the arithmetic is the full-grid step's own kernels, so the decomposed
  * step gives the values cs_ch_step gives.
- * Without transposes, when every band is a whole number of the y lines' chunks (the spike
- * method's partition, cs_ch_partition): steps 4-6 become
+ * Without transposes, when every band is a whole number of the y lines' chunks (the partition of
+ * the line solves, cs_ch_partition): steps 4-6 become
  *   4'. cs_ch_band_ycols_local: the chunk-local solves of the band's chunks of every column, and
  *       their end values (4 per column and chunk);
  *   5'. an all-gather of the end values of every band, in chunk order (4 * chunks * n values, the
  *       only data the ranks exchange for the y lines);
- *   6'. cs_ch_band_ycols_correct: the spike correction of the band's chunks, giving v.
+ *   6'. cs_ch_band_ycols_correct: the correction of the band's chunks, giving v.
  *
  * cs_ch_band_create: desc as for cs_ch_create (boundary CS_CH_PERIODIC or CS_CH_NOFLUX; the
  *   partition is the one cs_ch_create picks for the same description); rows = the band's row
  *   count, a multiple of 32 in [32, n].  The plan owns the line solver's tables and an FP64
- *   scratch of rows x n, plus 4 * chunks * rows values.
+ *   scratch of rows x n, plus 8.5 * chunks * n values.
  * Padded fields: (rows + 4) x n values of the storage type, row-major; rows 0-1 hold the two rows
  *   above the band, rows 2 .. rows+1 the band, rows rows+2 .. rows+3 the two rows below.
  * cs_ch_band_rhs(d_prev, d_cur): padded C^{n-1}, C^n (halos filled) -> d_rhs (rows x n FP64; may be
@@ -393,7 +393,7 @@ int cs_ch_partition(const cs_ch_desc* desc, int32_t* chunks, int32_t* chunk_len)
  * column (rows a whole number of chunks; CS_EINVAL otherwise), in two phases:
  * cs_ch_band_ycols_local(d_in, d_ends): d_in the band's rows x n FP64 values of w (the x solves'
  *   result); solves each chunk of each column locally into the plan's scratch and writes the
- *   chunks' end values to d_ends (device, 4 * (rows / chunk_len) * n FP64, chunk-major).
+ *   chunks' end values (of the forward and backward recursions) to d_ends (device, 4 * (rows / chunk_len) * n FP64, chunk-major).
  * cs_ch_band_ycols_correct(d_ends_all, d_v): d_ends_all the end values of all chunks of the line,
  *   in chunk order (every band's d_ends, gathered); writes v (rows x n FP64) for the band's rows,
  *   which cs_ch_band_update turns into C^{n+1}.  Uses the scratch phase 1 filled: no

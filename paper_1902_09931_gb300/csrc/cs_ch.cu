@@ -16,36 +16,44 @@
 // arithmetic there would lose every digit of C at n = 4096 (a = 1.8e5).
 //
 // Line solves (the paper uses cuPentBatch with the periodic corners treated as in Navon's
-// PENT).  Here each periodic line of length n is cut into P chunks of m = n / P points; since
-// every chunk block A (m x m pentadiagonal Toeplitz) and every coupling are identical for all
-// lines, chunks and steps, the library precomputes once:
-//   - the LU factors of A,
-//   - the spikes S_L = A^{-1} E_L, S_R = A^{-1} E_R (responses to the two values on each side),
-//   - the inverse of the block-circulant 4P x 4P system for the chunk-end values.
-// Per sweep, phase 1 solves A g = b on every (line, chunk) independently and records g at the
-// chunk ends; phase 2 forms the two end values of each neighbouring chunk from the recorded
-// ends (16 P FMAs) and corrects x = g - S_L t_{p-1} - S_R h_{p+1}.  This is exact (up to
-// rounding) and gives n * P independent threads instead of n sequential lines.
+// PENT): cs_penta.cuh's factored recursions in 64-bit fixed point, every line cut into P chunks of
+// m = n / P points, one thread per (line, chunk).  Two launches a step, one along the rows and one along
+// the columns with the update fused; each holds its lines in shared memory, so the field is read
+// once and written once.  4096^2, FP64 storage, periodic: rows 160 us (DRAM floor 39 us, bound by the
+// integer pipes at ~250 issue slots of a scheduler per 32 points), columns 223 us (floor 59 us), the step
+// 0.857 -> 0.582 ms; 1024^2 110 -> 63 us.
 //
 // No-flux boundaries (cs_ch_desc.boundary = CS_CH_NOFLUX): the same step on a cell-centred
 // grid whose stencils read ghost cells by even reflection.  Reflection commutes with the
 // 5-point Laplacian, so the factored right-hand side holds unchanged -- only the tile loader
-// mirrors indices instead of wrapping them.  The line operator is non-cyclic, I + a D4 with the
-// reflected fourth difference (first rows (1+2a, -3a, a), (-3a, 1+6a, -4a, a)): the first and
-// last chunks of a line get their own LU factors and spikes, the couplings are the same, and the
-// chunk-end system is inverted as a dense 4P x 4P matrix (no longer block-circulant; applying it
-// still takes 16 P FMAs per chunk).
+// mirrors indices instead of wrapping them.  The line operator is I + a D4 with the reflected fourth
+// difference (first rows (1+2a, -3a, a), (-3a, 1+6a, -4a, a)): the recursions are the same, only the
+// states entering the first and last chunks follow from the mirror conditions instead of the wrap.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
+
+#include <cooperative_groups.h>
 
 #include "cs_digits.cuh"
 #include "cs_internal.h"
+#include "cs_penta.cuh"
 
 namespace cs {
+
+// The line solver of a plan (cs_penta.cuh): constants, device tables (mats, then the table rows, then
+// the bias terms, in one allocation), and the scratch of the kernels that work from global memory (end
+// values, states, scale marks), allocated only for plans that run them.
+struct Lines {
+  pn::Par par;
+  double* tables;
+  double* scratch;
+  int P, m;
+};
 
 struct CHPlan {
   int64_t n;
@@ -56,10 +64,8 @@ struct CHPlan {
   int iprev, icur, inext;
   int64_t steps;
   double* A;         // n*n scratch (RHS, then w)
-  double* B;         // n*n scratch (local solutions g)
-  double* bnd;       // 4 * P * n chunk-end values
-  double* coef;      // 9 * m line-solve coefficients
-  double* K;         // P * 16 block-circulant inverse
+  double* B;         // n*n scratch (local solutions of lines too long for shared memory; coarsening)
+  Lines lines;       // the line solver's constants, tables and (long lines only) scratch
   double* partials;  // 2 per RHS block
   double* inv;       // 2 per step (device)
   int64_t inv_cap;
@@ -218,10 +224,6 @@ __device__ __forceinline__ double i128_to_double(__int128 v) {
   return neg ? -r : r;
 }
 
-template <typename T> __device__ __forceinline__ void store_as(T* p, double v);
-template <> __device__ __forceinline__ void store_as<double>(double* p, double v) { *p = v; }
-template <> __device__ __forceinline__ void store_as<float>(float* p, double v) { *p = narrow_rn(v); }
-
 __device__ __forceinline__ int wrapn(int64_t k, int64_t n) {
   return static_cast<int>(k < 0 ? k + n : (k >= n ? k - n : k));
 }
@@ -229,9 +231,6 @@ __device__ __forceinline__ int wrapn(int64_t k, int64_t n) {
 __device__ __forceinline__ int mirrorn(int64_t k, int64_t n) {
   return static_cast<int>(k < 0 ? -1 - k : (k >= n ? 2 * n - 1 - k : k));
 }
-// line-solve chunk type: bit 0 the line's first chunk, bit 1 its last (no-flux tables)
-__host__ __device__ __forceinline__ int chunk_type(int p, int P) { return (p == 0 ? 1 : 0) | (p == P - 1 ? 2 : 0); }
-
 // 128-bit shuffle (two 64-bit halves)
 __device__ __forceinline__ __int128 shfl_down_i128(__int128 v, int off) {
   const unsigned long long lo = __shfl_down_sync(0xffffffffu, static_cast<unsigned long long>(v), off);
@@ -611,454 +610,426 @@ __global__ void k_reduce_final(const double* __restrict__ partials, int nblocks,
   }
 }
 
-// 32-byte global accesses (one whole sector per thread and instruction)
-__device__ __forceinline__ void ld_v4(const double* p, double& a, double& b, double& c, double& d) {
-  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p) : "memory");
-}
-__device__ __forceinline__ void st_v4(double* p, double a, double b, double c, double d) {
-  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
-}
+// ---- line solves (cs_penta.cuh) ---------------------------------------------------------------------
+// A line's tables on the device: the table rows and the bias terms of phase 2, and the 8 P
+// matrices of the chunk scan.
+struct LineTab {
+  const pn::TabRow* tab;
+  const uint64_t* base;
+  const double* mats;
+};
 
-// A batch of kU line elements starting at `at` (element stride es): when the line is contiguous
-// (rows; `at` is then a multiple of kU) 32-byte accesses where both buffers of the kernel are
-// 32-byte aligned (wide), else 16-byte ones; strided scalars for the other direction.  A thread of
-// the row solves walks its own row, so a warp's access touches 32 rows: the 32-byte form fetches a
-// whole sector per thread and instruction.
-template <typename IT, bool CONTIG>
-__device__ __forceinline__ void load_batch(const IT* __restrict__ p, int64_t at, int64_t es, double (&v)[8],
-                                           bool wide = false) {
-  if constexpr (CONTIG && sizeof(IT) == 8) {
-    if (wide) {
-      ld_v4(p + at, v[0], v[1], v[2], v[3]);
-      ld_v4(p + at + 4, v[4], v[5], v[6], v[7]);
-      return;
-    }
+// Accessors of one thread's chunk: 8 consecutive 64-bit words.
+struct AccRow {  // words in a row, 16-byte aligned (shared memory)
+  uint64_t* p;
+  __device__ __forceinline__ void load8(int k, uint64_t (&v)[8]) const {
 #pragma unroll
     for (int u = 0; u < 8; u += 2) {
-      const double2 d = *reinterpret_cast<const double2*>(p + at + u);
+      const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(p + k + u);
       v[u] = d.x;
       v[u + 1] = d.y;
     }
-  } else if constexpr (CONTIG) {
-#pragma unroll
-    for (int u = 0; u < 8; u += 4) {
-      const float4 f = *reinterpret_cast<const float4*>(p + at + u);
-      v[u] = widen(f.x); v[u + 1] = widen(f.y); v[u + 2] = widen(f.z); v[u + 3] = widen(f.w);
-    }
-  } else {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = widen(p[at + u * es]);
   }
-}
-template <bool CONTIG>
-__device__ __forceinline__ void store_batch(double* __restrict__ p, int64_t at, int64_t es, const double (&v)[8],
-                                            bool wide = false) {
-  if constexpr (CONTIG) {
-    if (wide) {
-      st_v4(p + at, v[0], v[1], v[2], v[3]);
-      st_v4(p + at + 4, v[4], v[5], v[6], v[7]);
-      return;
-    }
+  __device__ __forceinline__ void store8(int k, const uint64_t (&v)[8]) const {
 #pragma unroll
-    for (int u = 0; u < 8; u += 2) *reinterpret_cast<double2*>(p + at + u) = make_double2(v[u], v[u + 1]);
-  } else {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) p[at + u * es] = v[u];
+    for (int u = 0; u < 8; u += 2) *reinterpret_cast<ulonglong2*>(p + k + u) = make_ulonglong2(v[u], v[u + 1]);
   }
-}
+};
+struct AccStride {  // words es apart (shared or global memory)
+  uint64_t* p;
+  int64_t es;
+  __device__ __forceinline__ void load8(int k, uint64_t (&v)[8]) const {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = p[(k + u) * es];
+  }
+  __device__ __forceinline__ void store8(int k, const uint64_t (&v)[8]) const {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) p[(k + u) * es] = v[u];
+  }
+};
+template <int ES>
+struct AccCols {  // ES columns interleaved (shared memory)
+  uint64_t* p;
+  __device__ __forceinline__ void load8(int k, uint64_t (&v)[8]) const {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = p[(k + u) * ES];
+  }
+  __device__ __forceinline__ void store8(int k, const uint64_t (&v)[8]) const {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) p[(k + u) * ES] = v[u];
+  }
+};
 
-// Phase 1: A g = b on chunk p of a line (LU forward then backward), g over the scratch.
-// Coefficients (negated / pre-scaled): nl1, nl2, dinv, nu1, nu2 at coef[0..5m).  Elements are
-// processed in register batches of kU so that a batch's loads are in flight together.
-// NF: no-flux tables, one set of 9 m coefficients per chunk type.
-template <typename IT, bool CONTIG, bool NF>
-__global__ void __launch_bounds__(kSolveThreads)
-    k_solve_local(const IT* __restrict__ in, double* __restrict__ G, double* __restrict__ bnd,
-                  const double* __restrict__ coef, int64_t n, int P, int m, int64_t line_stride,
-                  int64_t elem_stride, int p0 = 0, int Pl = -1) {
-  // chunks p0 .. p0 + Pl - 1 of every line (all P of them by default); the data, G and bnd hold
-  // only those, indexed from the first
-  if (Pl < 0) Pl = P;
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n * Pl) return;
-  const int64_t line = t % n;
-  const int pl = static_cast<int>(t / n);
-  const int p = p0 + pl;
-  const int64_t es = CONTIG ? 1 : elem_stride;
-  if constexpr (NF) coef += static_cast<int64_t>(chunk_type(p, P)) * 9 * m;
-  const double* nl1 = coef;
-  const double* nl2 = coef + m;
-  const double* dinv = coef + 2 * m;
-  const double* nu1 = coef + 3 * m;
-  const double* nu2 = coef + 4 * m;
-  const int64_t base = line * line_stride + static_cast<int64_t>(pl) * m * es;
-  // rows: base is a multiple of kU elements (m and the line stride are multiples of 64)
-  const bool wide = CONTIG && sizeof(IT) == 8 &&
-                    ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(G)) & 31u) == 0;
-  double y1 = 0.0, y2 = 0.0;
-  for (int k0 = 0; k0 < m; k0 += kU) {
-    double v[kU];
-    load_batch<IT, CONTIG>(in, base + k0 * es, es, v, wide);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const double y = fma(__ldg(nl1 + k0 + u), y1, fma(__ldg(nl2 + k0 + u), y2, v[u]));
-      v[u] = y;
-      y2 = y1;
-      y1 = y;
+// The states entering chunk p of a line from all its chunks' end values: inclusive scans over the
+// chunks with the recursion's own matrices, forward states then backward ones.  Every thread of the
+// block calls it, P threads per line; sh: P double2 of the line.  The order of operations is
+// reduce_host's.
+template <bool NF>
+__device__ __forceinline__ void reduce_states(const pn::Par& q, const double* __restrict__ mats, int P, int p,
+                                              double2* sh, const double (&ends)[4], double (&st)[4]) {
+  const bool cyclic = !NF && q.cyclic;
+  auto scan = [&](bool fwd, double& a, double& b) {
+#pragma unroll 1
+    for (int l = 0; (1 << l) < P && l < q.levels; ++l) {
+      int o = fwd ? p - (1 << l) : p + (1 << l);
+      if (cyclic) o = o < 0 ? o + P : (o >= P ? o - P : o);
+      sh[p] = make_double2(a, b);
+      __syncthreads();
+      if (o >= 0 && o < P) {
+        const double2 v = sh[o];
+        pn::mv_add(q.Ml[l], v.x, v.y, a, b, a, b);
+      }
+      __syncthreads();
     }
-    store_batch<CONTIG>(G, base + k0 * es, es, v, wide);
-  }
-  double g1 = 0.0, g2 = 0.0, g_last = 0.0, g_last2 = 0.0;
-  for (int k0 = m - kU; k0 >= 0; k0 -= kU) {
-    double v[kU];
-    load_batch<double, CONTIG>(G, base + k0 * es, es, v, wide);
-#pragma unroll
-    for (int u = kU - 1; u >= 0; --u) {
-      const int k = k0 + u;
-      const double g = fma(__ldg(nu1 + k), g1, fma(__ldg(nu2 + k), g2, v[u] * __ldg(dinv + k)));
-      v[u] = g;
-      g2 = g1;
-      g1 = g;
-    }
-    if (k0 == m - kU) {
-      g_last2 = v[kU - 2];
-      g_last = v[kU - 1];
-    }
-    store_batch<CONTIG>(G, base + k0 * es, es, v, wide);
-  }
-  // chunk-end values: k = 0, 1 are g1, g2 after the loop; k = m-2, m-1 kept from the first batch
-  double* b = bnd + static_cast<int64_t>(pl) * 4 * n + line;
-  b[0] = g1;
-  b[n] = g2;
-  b[2 * n] = g_last2;
-  b[3 * n] = g_last;
-}
-
-// Phase 2: end values of the neighbouring chunks from the block-circulant inverse (staged in
-// shared memory), then the spike correction.  MODE 0 writes w (FP64); MODE 1 writes
-// C^{n+1} = 2 C^n - C^{n-1} + x (for FP32 storage 2 C^n - C^{n-1} is formed in FP32: its one
-// rounding, <= 2^-24 |Cbar|, is of the size of the rounding of the stored result).
-// NF: no-flux tables (per chunk type) and the dense 4P x 4P chunk-end inverse, read through the
-// read-only cache; the line's first chunk has no left neighbour, its last no right one.
-template <int MODE, typename T, bool CONTIG, bool NF>
-__global__ void __launch_bounds__(kSolveThreads)
-    k_solve_correct(const double* __restrict__ G, const double* __restrict__ bnd,
-                    const double* __restrict__ coef, const double* __restrict__ K, int64_t n, int P,
-                    int m, int64_t line_stride, int64_t elem_stride, double* __restrict__ w_out,
-                    const T* __restrict__ cur, const T* __restrict__ prev, T* __restrict__ next, int p0 = 0,
-                    int Pl = -1) {
-  // chunks p0 .. p0 + Pl - 1 of every line (all P by default): G, w_out and the fields hold only
-  // those, indexed from the first; bnd holds the end values of all P chunks
-  extern __shared__ double sK[];
-  if (Pl < 0) Pl = P;
-  if constexpr (!NF) {
-    for (int i = threadIdx.x; i < 16 * P; i += blockDim.x) sK[i] = K[i];
+    sh[p] = make_double2(a, b);
+    __syncthreads();
+  };
+  // a value that is not finite reaches every chunk of its line, as it would with every level
+  auto finite = [](double x) { return ((pn::hi32(pn::dbits(x)) >> 20) & 0x7ffu) != 0x7ffu; };
+  const bool own = finite(ends[0]) && finite(ends[1]) && finite(ends[2]) && finite(ends[3]);
+  const bool broken = __syncthreads_or(!own);  // uniform over the block
+  bool line_broken = false;
+  if (broken) {
+    sh[p] = make_double2(own ? 0.0 : 1.0, 0.0);
+    __syncthreads();
+    for (int k = 0; k < P; ++k) line_broken = line_broken || sh[k].x != 0.0;
     __syncthreads();
   }
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= n * Pl) return;
-  const int64_t line = t % n;
-  const int pl = static_cast<int>(t / n);
-  const int p = p0 + pl;
-  const int64_t es = CONTIG ? 1 : elem_stride;
-  double t0 = 0.0, t1 = 0.0, h0 = 0.0, h1 = 0.0;
+  double a = ends[0], b = ends[1];
+  scan(true, a, b);
+  const double2 last = sh[P - 1];
+  const int o = p > 0 ? p - 1 : P - 1;
+  const double2 before = sh[o];
+  double y0 = 0.0, y1 = 0.0;
+  if (cyclic) {
+    y0 = before.x;
+    y1 = before.y;
+  } else if constexpr (!NF) {
+    double t0, t1;
+    pn::mv_add(q.C, last.x, last.y, 0.0, 0.0, t0, t1);
+    pn::mv_add(mats + 8 * o, t0, t1, before.x, before.y, y0, y1);
+  } else if (p > 0) {
+    y0 = before.x;
+    y1 = before.y;
+  }
+  __syncthreads();
+  pn::mv_add(q.R, y0, y1, ends[2], ends[3], a, b);
   if constexpr (NF) {
-    coef += static_cast<int64_t>(chunk_type(p, P)) * 9 * m;
-    const int64_t N4 = 4 * static_cast<int64_t>(P);
-    const bool left = p > 0, right = p + 1 < P;
-    const double* Kt = left ? K + (4 * static_cast<int64_t>(p - 1) + 2) * N4 : K;  // rows of x_{p-1}[m-2], [m-1]
-    const double* Kh = right ? K + (4 * static_cast<int64_t>(p + 1)) * N4 : K;     // rows of x_{p+1}[0], [1]
-    for (int q = 0; q < P; ++q) {
-      const double* b = bnd + static_cast<int64_t>(q) * 4 * n + line;
-      const double g0 = b[0], g1 = b[n], g2 = b[2 * n], g3 = b[3 * n];
-      if (left) {
-        const double* r2 = Kt + 4 * q;
-        const double* r3 = r2 + N4;
-        t0 = fma(__ldg(r2), g0, fma(__ldg(r2 + 1), g1, fma(__ldg(r2 + 2), g2, fma(__ldg(r2 + 3), g3, t0))));
-        t1 = fma(__ldg(r3), g0, fma(__ldg(r3 + 1), g1, fma(__ldg(r3 + 2), g2, fma(__ldg(r3 + 3), g3, t1))));
-      }
-      if (right) {
-        const double* r0 = Kh + 4 * q;
-        const double* r1 = r0 + N4;
-        h0 = fma(__ldg(r0), g0, fma(__ldg(r0 + 1), g1, fma(__ldg(r0 + 2), g2, fma(__ldg(r0 + 3), g3, h0))));
-        h1 = fma(__ldg(r1), g0, fma(__ldg(r1 + 1), g1, fma(__ldg(r1 + 2), g2, fma(__ldg(r1 + 3), g3, h1))));
-      }
+    if (p == P - 1) {
+      double w0, w1;
+      pn::mv_add(q.V, last.x, last.y, 0.0, 0.0, w0, w1);
+      pn::mv_add(q.M, w0, w1, a, b, a, b);
     }
+  }
+  scan(false, a, b);
+  const double2 first = sh[0];
+  const int nx = p + 1 < P ? p + 1 : 0;
+  const double2 after = sh[nx];
+  double z0, z1;
+  if (cyclic) {
+    st[2] = after.x;
+    st[3] = after.y;
+  } else if constexpr (!NF) {
+    pn::mv_add(q.C, first.x, first.y, 0.0, 0.0, z0, z1);
+    pn::mv_add(mats + 8 * (P - 1 - nx), z0, z1, after.x, after.y, st[2], st[3]);
   } else {
-    const int pm = (p + P - 1) % P, pp = (p + 1) % P;
-    for (int q = 0; q < P; ++q) {
-      const double* b = bnd + static_cast<int64_t>(q) * 4 * n + line;
-      const double g0 = b[0], g1 = b[n], g2 = b[2 * n], g3 = b[3 * n];
-      const double* Kt = sK + ((pm - q + P) % P) * 16;  // K_{(p-1)-q}: rows 2, 3 give t_{p-1}
-      const double* Kh = sK + ((pp - q + P) % P) * 16;  // K_{(p+1)-q}: rows 0, 1 give h_{p+1}
-      t0 = fma(Kt[8], g0, fma(Kt[9], g1, fma(Kt[10], g2, fma(Kt[11], g3, t0))));
-      t1 = fma(Kt[12], g0, fma(Kt[13], g1, fma(Kt[14], g2, fma(Kt[15], g3, t1))));
-      h0 = fma(Kh[0], g0, fma(Kh[1], g1, fma(Kh[2], g2, fma(Kh[3], g3, h0))));
-      h1 = fma(Kh[4], g0, fma(Kh[5], g1, fma(Kh[6], g2, fma(Kh[7], g3, h1))));
-    }
-  }
-  const double* sl0 = coef + 5 * m;
-  const double* sl1 = coef + 6 * m;
-  const double* sr0 = coef + 7 * m;
-  const double* sr1 = coef + 8 * m;
-  const int64_t base = line * line_stride + static_cast<int64_t>(pl) * m * es;
-  const bool wide = CONTIG && MODE == 0 &&
-                    ((reinterpret_cast<uintptr_t>(G) | reinterpret_cast<uintptr_t>(w_out)) & 31u) == 0;
-  for (int k0 = 0; k0 < m; k0 += kU) {
-    double x[kU];
-    load_batch<double, CONTIG>(G, base + k0 * es, es, x, wide);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int k = k0 + u;
-      x[u] = fma(-__ldg(sl0 + k), t0, fma(-__ldg(sl1 + k), t1,
-             fma(-__ldg(sr0 + k), h0, fma(-__ldg(sr1 + k), h1, x[u]))));
-    }
-    if constexpr (MODE == 0) {
-      store_batch<CONTIG>(w_out, base + k0 * es, es, x, wide);
+    pn::mv_add(q.Z, first.x, first.y, 0.0, 0.0, z0, z1);
+    if (p > 0) pn::mv_add(mats + 8 * (p - 1), z0, z1, y0, y1, y0, y1);
+    else { y0 = z0; y1 = z1; }
+    if (p + 1 < P) {
+      pn::mv_add(mats + 8 * nx + 4, z0, z1, after.x, after.y, st[2], st[3]);
     } else {
-      // next holds Cbar = 2 C^n - C^{n-1}, written there by this step's right-hand side kernel
-      // (FP32 storage: formed in FP32, one rounding of the size of the result's own); C^{n+1} =
-      // Cbar + v replaces it element by element
-      if constexpr (sizeof(T) == 4) {
-        // one FP64 add of x, then the round-to-nearest-even narrowing on the integer pipe (this
-        // kernel is FP64-bound, and a conversion instruction would take an FP64 issue slot)
-        float cb[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) cb[u] = next[base + (k0 + u) * es];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) next[base + (k0 + u) * es] = narrow_rn(widen(cb[u]) + x[u]);
-      } else {
-        double cb[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) cb[u] = next[base + (k0 + u) * es];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) store_as<T>(next + base + (k0 + u) * es, cb[u] + x[u]);
-      }
+      double t0, t1;
+      pn::mv_add(mats + 8 * (P - 1), z0, z1, last.x, last.y, t0, t1);
+      pn::mv_add(q.V, t0, t1, 0.0, 0.0, st[2], st[3]);
     }
   }
+  st[0] = y0;
+  st[1] = y1;
+  if (line_broken) st[0] = st[1] = st[2] = st[3] = pn::from_bits(0x7ff8000000000000ull);
 }
 
-// ---- host-side precomputation ---------------------------------------------------------------
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory"); }
 
-// LU of the m x m pentadiagonal Toeplitz block, rows (a, -4a, 1+6a, -4a, a), no pivoting
-// (the block is symmetric positive definite).  L unit lower with bands l1, l2; U with d, u1, u2.
-void block_lu(int m, double a, std::vector<double>& l1, std::vector<double>& l2,
-              std::vector<double>& d, std::vector<double>& u1, std::vector<double>& u2) {
-  l1.assign(m, 0.0); l2.assign(m, 0.0); d.assign(m, 0.0); u1.assign(m, 0.0); u2.assign(m, 0.0);
-  for (int k = 0; k < m; ++k) {
-    const double sub2 = k >= 2 ? a : 0.0;
-    const double sub1 = k >= 1 ? -4.0 * a : 0.0;
-    l2[k] = k >= 2 ? sub2 / d[k - 2] : 0.0;
-    l1[k] = k >= 1 ? (sub1 - (k >= 2 ? l2[k] * u1[k - 2] : 0.0)) / d[k - 1] : 0.0;
-    d[k] = 1.0 + 6.0 * a - (k >= 2 ? l2[k] * u2[k - 2] : 0.0) - (k >= 1 ? l1[k] * u1[k - 1] : 0.0);
-    u1[k] = k + 1 < m ? -4.0 * a - (k >= 1 ? l1[k] * u2[k - 1] : 0.0) : 0.0;
-    u2[k] = k + 2 < m ? a : 0.0;
+// The table rows of phase 2, the same for every thread: from shared memory in the kernels that stage
+// them (from global memory their latency bounded phase 2: 108 cycles a point and warp scheduler,
+// 62 from shared memory), through the read-only cache otherwise.
+struct TabShared {
+  const ulonglong2* t;
+  const uint64_t* b;
+  __device__ __forceinline__ void row(int k, uint64_t (&v)[4], uint64_t& base) const {
+    const ulonglong2 x = t[2 * k], y = t[2 * k + 1];
+    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+    base = b[k];
   }
+};
+struct TabGlobal {
+  const ulonglong2* t;
+  const unsigned long long* b;
+  __device__ __forceinline__ explicit TabGlobal(const LineTab& lt)
+      : t(reinterpret_cast<const ulonglong2*>(lt.tab)), b(reinterpret_cast<const unsigned long long*>(lt.base)) {}
+  __device__ __forceinline__ void row(int k, uint64_t (&v)[4], uint64_t& base) const {
+    const ulonglong2 x = __ldg(t + 2 * k), y = __ldg(t + 2 * k + 1);
+    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+    base = __ldg(b + k);
+  }
+};
+constexpr int kTabBytes = 40;  // per point of a chunk
+
+// Starts the copy of the tables to shared memory (16-byte aligned, kTabBytes m): rows, then bias terms
+// (m is a multiple of 8).  The caller waits for it with its other copies.
+__device__ __forceinline__ TabShared stage_tables(uint64_t* to, const LineTab& lt, int m) {
+  for (int i = threadIdx.x; i < 2 * m; i += blockDim.x) cp_async16(to + 2 * i, reinterpret_cast<const uint64_t*>(lt.tab) + 2 * i);
+  for (int i = threadIdx.x; i < m / 2; i += blockDim.x) cp_async16(to + 4 * m + 2 * i, lt.base + 2 * i);
+  return {reinterpret_cast<const ulonglong2*>(to), to + 4 * m};
 }
 
-// LU (no pivoting) of an m x m pentadiagonal block given by its bands: sub2[k] = A(k, k-2),
-// sub1[k] = A(k, k-1), diag[k], sup1[k] = A(k, k+1), sup2[k] = A(k, k+2).
-void penta_lu(int m, const std::vector<double>& sub2, const std::vector<double>& sub1,
-              const std::vector<double>& diag, const std::vector<double>& sup1,
-              const std::vector<double>& sup2, std::vector<double>& l1, std::vector<double>& l2,
-              std::vector<double>& d, std::vector<double>& u1, std::vector<double>& u2) {
-  l1.assign(m, 0.0); l2.assign(m, 0.0); d.assign(m, 0.0); u1.assign(m, 0.0); u2.assign(m, 0.0);
-  for (int k = 0; k < m; ++k) {
-    l2[k] = k >= 2 ? sub2[k] / d[k - 2] : 0.0;
-    l1[k] = k >= 1 ? (sub1[k] - (k >= 2 ? l2[k] * u1[k - 2] : 0.0)) / d[k - 1] : 0.0;
-    d[k] = diag[k] - (k >= 2 ? l2[k] * u2[k - 2] : 0.0) - (k >= 1 ? l1[k] * u1[k - 1] : 0.0);
-    u1[k] = k + 1 < m ? sup1[k] - (k >= 1 ? l1[k] * u2[k - 1] : 0.0) : 0.0;
-    u2[k] = k + 2 < m ? sup2[k] : 0.0;
-  }
-}
-
-void block_solve(int m, const std::vector<double>& l1, const std::vector<double>& l2,
-                 const std::vector<double>& d, const std::vector<double>& u1,
-                 const std::vector<double>& u2, std::vector<double>& x) {
-  for (int k = 0; k < m; ++k) {
-    if (k >= 1) x[k] -= l1[k] * x[k - 1];
-    if (k >= 2) x[k] -= l2[k] * x[k - 2];
-  }
-  for (int k = m - 1; k >= 0; --k) {
-    if (k + 1 < m) x[k] -= u1[k] * x[k + 1];
-    if (k + 2 < m) x[k] -= u2[k] * x[k + 2];
-    x[k] /= d[k];
-  }
-}
-
-// Gauss-Jordan inverse with partial pivoting (dense, small), then two steps of Newton refinement
-// K <- K + K (I - R K) whose residual I - R K is accumulated with error-free products and sums
-// (FMA and TwoSum), so it is exact to rounding although it is far smaller than R K: the
-// chunk-end system's condition number grows with a, and the plain inverse's rounding (~cond * eps)
-// went straight into every corrected value (the solver's backward error was 3.9e-13 of
-// (1 + 16 a) |x| at n = 4096 with no-flux boundaries; refined it is 2.6e-15).
-bool invert(int N, std::vector<double>& Min, std::vector<double>& inv) {
-  const std::vector<double> R = Min;
-  std::vector<double>& M = Min;
-  inv.assign(static_cast<size_t>(N) * N, 0.0);
-  for (int i = 0; i < N; ++i) inv[static_cast<size_t>(i) * N + i] = 1.0;
-  for (int c = 0; c < N; ++c) {
-    int piv = c;
-    for (int r = c + 1; r < N; ++r)
-      if (std::fabs(M[static_cast<size_t>(r) * N + c]) > std::fabs(M[static_cast<size_t>(piv) * N + c])) piv = r;
-    if (M[static_cast<size_t>(piv) * N + c] == 0.0) return false;
-    if (piv != c)
-      for (int k = 0; k < N; ++k) {
-        std::swap(M[static_cast<size_t>(c) * N + k], M[static_cast<size_t>(piv) * N + k]);
-        std::swap(inv[static_cast<size_t>(c) * N + k], inv[static_cast<size_t>(piv) * N + k]);
+// Phase 2 on a thread's chunk: every word of s (W at scale mark ew) becomes x, as a double's bits.
+template <class Tab, class Acc>
+__device__ __forceinline__ void correct_chunk(const pn::Par& q, const Tab& tab, const Acc& s, int m, int ew,
+                                              const double (&st)[4]) {
+  pn::Corr c;
+  if (pn::corr_setup(q, ew, st, c)) {
+    for (int k0 = 0; k0 < m; k0 += 8) {
+      uint64_t v[8];
+      s.load8(k0, v);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        uint64_t t[4], b;
+        tab.row(k0 + u, t, b);
+        v[u] = pn::dbits(pn::from_fixed(pn::corr_point(c, v[u], t, b), c.eo));
       }
-    const double s = 1.0 / M[static_cast<size_t>(c) * N + c];
-    for (int k = 0; k < N; ++k) {
-      M[static_cast<size_t>(c) * N + k] *= s;
-      inv[static_cast<size_t>(c) * N + k] *= s;
+      s.store8(k0, v);
     }
-    for (int r = 0; r < N; ++r) {
-      if (r == c) continue;
-      const double f = M[static_cast<size_t>(r) * N + c];
-      if (f == 0.0) continue;
-      for (int k = 0; k < N; ++k) {
-        M[static_cast<size_t>(r) * N + k] -= f * M[static_cast<size_t>(c) * N + k];
-        inv[static_cast<size_t>(r) * N + k] -= f * inv[static_cast<size_t>(c) * N + k];
-      }
-    }
+    return;
   }
-  std::vector<double> E(static_cast<size_t>(N) * N), C(static_cast<size_t>(N) * N);
-  for (int it = 0; it < 2; ++it) {
-    for (int r = 0; r < N; ++r)
-      for (int c = 0; c < N; ++c) {  // E = I - R K, each entry as an unevaluated sum hi + lo
-        double hi = r == c ? 1.0 : 0.0, lo = 0.0;
-        for (int k = 0; k < N; ++k) {
-          const double p = -R[static_cast<size_t>(r) * N + k] * inv[static_cast<size_t>(k) * N + c];
-          const double pe = std::fma(-R[static_cast<size_t>(r) * N + k], inv[static_cast<size_t>(k) * N + c], -p);
-          const double t = hi + p, bb = t - hi;
-          lo += (hi - (t - bb)) + (p - bb) + pe;
-          hi = t;
+#pragma unroll 1
+  for (int k0 = 0; k0 < m; k0 += 8) {
+    uint64_t v[8];
+    s.load8(k0, v);
+#pragma unroll 1
+    for (int u = 0; u < 8; ++u) {
+      uint64_t t[4], b;
+      tab.row(k0 + u, t, b);
+      v[u] = pn::dbits(pn::corr_native(q, ew, v[u], t, st));
+    }
+    s.store8(k0, v);
+  }
+}
+
+// C^{n+1} = Cbar + v of one point: next holds Cbar = 2 C^n - C^{n-1}, written there by this step's
+// right-hand side kernel (FP32 storage: formed in FP32, one rounding of the size of the result's own).
+__device__ __forceinline__ double updated(double cbar, double v) { return cbar + v; }
+__device__ __forceinline__ float updated(float cbar, double v) { return narrow_rn(widen(cbar) + v); }
+
+// Whole lines in shared memory, both phases in one launch: the field is read once and written once.
+// Rows (COLS = 0): `lines` rows of n = P m values per block, one thread per (row, chunk); chunks padded
+// by 16 bytes so that the lanes' 16-byte accesses fall on different banks.
+template <bool NF>
+__global__ void __launch_bounds__(64)
+    k_line_rows(const double* __restrict__ in, double* __restrict__ out, const pn::Par q,
+                            const LineTab lt, int P, int m, int vec) {
+  extern __shared__ __align__(16) uint64_t sm[];
+  const int chunks = blockDim.x;  // lines * P
+  double2* sh = reinterpret_cast<double2*>(sm + static_cast<size_t>(chunks) * (m + 2));
+  const TabShared tab = stage_tables(reinterpret_cast<uint64_t*>(sh + chunks), lt, m);
+  const int64_t base = static_cast<int64_t>(blockIdx.x) * chunks * m;  // consecutive rows are one range
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+  const int lanes = min(32, static_cast<int>(blockDim.x) - 32 * warp);
+  for (int c = warp; c < chunks; c += nw) {
+    uint64_t* d = sm + c * (m + 2);
+    const double* g = in + base + static_cast<int64_t>(c) * m;
+    if (vec)
+      for (int k = 2 * lane; k < m; k += 2 * lanes) cp_async16(d + k, g + k);
+    else
+      for (int k = lane; k < m; k += lanes) cp_async8(d + k, g + k);
+  }
+  cp_async_wait();
+  __syncthreads();
+  const int p = threadIdx.x % P;
+  AccRow s{sm + threadIdx.x * (m + 2)};
+  double ends[4], st[4];
+  const int ew = pn::local_solve(q, s, s, m, ends);
+  reduce_states<NF>(q, lt.mats, P, p, sh + (threadIdx.x - p), ends, st);
+  correct_chunk(q, tab, s, m, ew, st);
+  __syncthreads();
+  for (int c = warp; c < chunks; c += nw) {
+    const double* d = reinterpret_cast<const double*>(sm + c * (m + 2));
+    double* g = out + base + static_cast<int64_t>(c) * m;
+    if (vec)
+      for (int k = 2 * lane; k < m; k += 2 * lanes) *reinterpret_cast<double2*>(g + k) = *reinterpret_cast<const double2*>(d + k);
+    else
+      for (int k = lane; k < m; k += lanes) g[k] = d[k];
+  }
+}
+
+// Columns: a cluster of CS blocks holds NC neighbouring columns, each block the n / CS rows of its
+// chunks, so that every row is an 8 NC-byte piece (whole 128-byte lines for NC = 16: with two columns
+// per block the 16-byte pieces alone took 0.35 ms at 4096^2) and a block still fits three to an
+// SM.  Threads are (chunk, column), columns fastest.  Each block forms the entering states of NC / CS of
+// the columns from all chunks' end values, read from and returned to the other blocks' shared
+// memory.  The update C^{n+1} = Cbar + v is fused into the write.
+template <int NC, typename T, bool NF>
+__global__ void __launch_bounds__(256)
+    k_line_cols(const double* __restrict__ in, T* __restrict__ next, int64_t n, const pn::Par q,
+                const LineTab lt, int P, int m, int vec) {
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) uint64_t sm[];
+  constexpr int H = NC / 2;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CS = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
+  const int Pc = P / CS, threads = static_cast<int>(blockDim.x);  // Pc * NC
+  // after the data: the scan's double2 per thread, then the end values (later the states), 4 per thread
+  double2* sh = reinterpret_cast<double2*>(sm + static_cast<size_t>(Pc) * (m + 1) * NC);
+  double* ex = reinterpret_cast<double*>(sh + threads);
+  const TabShared tab = stage_tables(reinterpret_cast<uint64_t*>(ex + 4 * threads), lt, m);
+  const int64_t x0 = static_cast<int64_t>(blockIdx.x / CS) * NC;
+  const int64_t row0 = static_cast<int64_t>(rank) * Pc * m;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (threads + 31) >> 5;
+  const int lanes = min(32, threads - 32 * warp);
+  for (int c = warp; c < Pc; c += nw) {
+    uint64_t* d = sm + c * (m + 1) * NC;
+    const double* g = in + (row0 + static_cast<int64_t>(c) * m) * n + x0;
+    for (int i = lane; i < m * H; i += lanes) cp_async16(d + 2 * i, g + static_cast<int64_t>(i / H) * n + 2 * (i % H));
+  }
+  cp_async_wait();
+  __syncthreads();
+  const int l = threadIdx.x % NC, c = threadIdx.x / NC;
+  AccCols<NC> s{sm + c * (m + 1) * NC + l};
+  double ends[4], st[4];
+  const int ew = pn::local_solve(q, s, s, m, ends);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) ex[j * threads + threadIdx.x] = ends[j];
+  cluster.sync();
+  {
+    // this block's share of the columns, P threads each: chunk p of column rl is thread
+    // (p % Pc) NC + rl of block p / Pc
+    const int rl = rank * (NC / CS) + threadIdx.x / P, p = threadIdx.x % P;
+    double* far = cluster.map_shared_rank(ex, p / Pc) + (p % Pc) * NC + rl;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ends[j] = far[j * threads];
+    reduce_states<NF>(q, lt.mats, P, p, sh + (threadIdx.x - p), ends, st);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) far[j * threads] = st[j];
+  }
+  cluster.sync();
+#pragma unroll
+  for (int j = 0; j < 4; ++j) st[j] = ex[j * threads + threadIdx.x];
+  correct_chunk(q, tab, s, m, ew, st);
+  __syncthreads();
+  for (int cc = warp; cc < Pc; cc += nw) {
+    const double* d = reinterpret_cast<const double*>(sm + cc * (m + 1) * NC);
+    T* g = next + (row0 + static_cast<int64_t>(cc) * m) * n + x0;
+    for (int i0 = lane; i0 < m * H; i0 += 4 * lanes) {  // four pieces in flight
+      using V = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
+      V cb[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = i0 + j * lanes;
+        if (i < m * H) {
+          const T* a = g + static_cast<int64_t>(i / H) * n + 2 * (i % H);
+          if (vec) cb[j] = *reinterpret_cast<const V*>(a);
+          else { cb[j].x = a[0]; cb[j].y = a[1]; }
         }
-        E[static_cast<size_t>(r) * N + c] = hi + lo;
       }
-    for (int r = 0; r < N; ++r)
-      for (int c = 0; c < N; ++c) {  // C = K E
-        double acc = 0.0;
-        for (int k = 0; k < N; ++k) acc = std::fma(inv[static_cast<size_t>(r) * N + k], E[static_cast<size_t>(k) * N + c], acc);
-        C[static_cast<size_t>(r) * N + c] = acc;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = i0 + j * lanes;
+        if (i < m * H) {
+          T* a = g + static_cast<int64_t>(i / H) * n + 2 * (i % H);
+          V r;
+          r.x = updated(cb[j].x, d[2 * i]);
+          r.y = updated(cb[j].y, d[2 * i + 1]);
+          if (vec) *reinterpret_cast<V*>(a) = r;
+          else { a[0] = r.x; a[1] = r.y; }
+        }
       }
-    for (size_t q = 0; q < C.size(); ++q) inv[q] += C[q];
+    }
   }
-  return true;
 }
 
-int build_tables_periodic(int64_t n, int P, double a, std::vector<double>& coef, std::vector<double>& K) {
-  const int m = static_cast<int>(n / P);
-  std::vector<double> l1, l2, d, u1, u2;
-  block_lu(m, a, l1, l2, d, u1, u2);
-  coef.assign(static_cast<size_t>(9) * m, 0.0);
-  for (int k = 0; k < m; ++k) {
-    coef[k] = -l1[k];
-    coef[m + k] = -l2[k];
-    coef[2 * m + k] = 1.0 / d[k];
-    coef[3 * m + k] = -u1[k] / d[k];
-    coef[4 * m + k] = -u2[k] / d[k];
-  }
-  // spikes: responses to the two values before (t) and after (h) the chunk
-  std::vector<double> s[4];
-  for (int c = 0; c < 4; ++c) s[c].assign(m, 0.0);
-  s[0][0] = a;                          // S_L column for x_{p-1}[m-2]
-  s[1][0] = -4.0 * a; s[1][1] = a;      // S_L column for x_{p-1}[m-1]
-  s[2][m - 2] = a; s[2][m - 1] = -4.0 * a;  // S_R column for x_{p+1}[0]
-  s[3][m - 1] = a;                      // S_R column for x_{p+1}[1]
-  for (int c = 0; c < 4; ++c) block_solve(m, l1, l2, d, u1, u2, s[c]);
-  for (int c = 0; c < 4; ++c)
-    for (int k = 0; k < m; ++k) coef[static_cast<size_t>(5 + c) * m + k] = s[c][k];
-  // block-circulant system for u_p = (x_p[0], x_p[1], x_p[m-2], x_p[m-1])
-  const int rows[4] = {0, 1, m - 2, m - 1};
-  const int N4 = 4 * P;
-  std::vector<double> R(static_cast<size_t>(N4) * N4, 0.0), Ri;
-  for (int i = 0; i < N4; ++i) R[static_cast<size_t>(i) * N4 + i] = 1.0;
-  for (int p = 0; p < P; ++p) {
-    const int pm = (p + P - 1) % P, pp = (p + 1) % P;
-    for (int r = 0; r < 4; ++r) {
-      const size_t row = static_cast<size_t>(4 * p + r) * N4;
-      R[row + 4 * pm + 2] += s[0][rows[r]];
-      R[row + 4 * pm + 3] += s[1][rows[r]];
-      R[row + 4 * pp + 0] += s[2][rows[r]];
-      R[row + 4 * pp + 1] += s[3][rows[r]];
-    }
-  }
-  if (!invert(N4, R, Ri)) return set_error(CS_EINVAL, "Cahn-Hilliard chunk system is singular");
-  K.assign(static_cast<size_t>(16) * P, 0.0);
-  for (int dd = 0; dd < P; ++dd)  // K_d = block (d, 0) of the inverse
-    for (int r = 0; r < 4; ++r)
-      for (int c = 0; c < 4; ++c) K[static_cast<size_t>(dd) * 16 + r * 4 + c] = Ri[static_cast<size_t>(4 * dd + r) * N4 + c];
-  return CS_OK;
+// Lines too long for shared memory, and the columns of a row band (whose chunks lie on several ranks):
+// the two phases as kernels over global memory, one thread per (line, chunk), with the same
+// functions, so the same values.  G holds W, scale the chunks' scale marks.
+__global__ void __launch_bounds__(kSolveThreads)
+    k_line_local(const double* __restrict__ in, uint64_t* __restrict__ G, double* __restrict__ bnd,
+                 int* __restrict__ scale, const pn::Par q, int64_t lines, int Pl, int m, int64_t line_stride,
+                 int64_t elem_stride) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= lines * Pl) return;
+  const int64_t line = t % lines, pl = t / lines;
+  const int64_t at = line * line_stride + pl * m * elem_stride;
+  const AccStride si{const_cast<uint64_t*>(reinterpret_cast<const uint64_t*>(in)) + at, elem_stride};
+  AccStride s{G + at, elem_stride};
+  double ends[4];
+  scale[pl * lines + line] = pn::local_solve(q, si, s, m, ends);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) bnd[(4 * pl + j) * lines + line] = ends[j];
 }
 
-// No-flux tables: for each chunk type t (bit 0: the line's first chunk, bit 1: its last) the LU
-// of the chunk block of L = I + a D4 (reflected rows at the line's ends) and the four spikes, at
-// coef[9 m t ..]; K = the dense inverse of the 4P x 4P chunk-end system, row-major.
-int build_tables_noflux(int64_t n, int P, double a, std::vector<double>& coef, std::vector<double>& K) {
-  const int m = static_cast<int>(n / P);
-  coef.assign(static_cast<size_t>(4) * 9 * m, 0.0);
-  std::vector<double> spk[4][4];  // [type][spike]
-  for (int t = 0; t < 4; ++t) {
-    std::vector<double> sub2(m, a), sub1(m, -4.0 * a), diag(m, 1.0 + 6.0 * a), sup1(m, -4.0 * a), sup2(m, a);
-    if (t & 1) {  // rows 0, 1 of the line: (1 + 2a, -3a, a), (-3a, 1 + 6a, -4a, a)
-      diag[0] = 1.0 + 2.0 * a;
-      sup1[0] = -3.0 * a;
-      sub1[1] = -3.0 * a;
-    }
-    if (t & 2) {  // rows n-2, n-1: mirrored
-      diag[m - 1] = 1.0 + 2.0 * a;
-      sub1[m - 1] = -3.0 * a;
-      sup1[m - 2] = -3.0 * a;
-    }
-    std::vector<double> l1, l2, d, u1, u2;
-    penta_lu(m, sub2, sub1, diag, sup1, sup2, l1, l2, d, u1, u2);
-    double* c = coef.data() + static_cast<size_t>(9) * m * t;
-    for (int k = 0; k < m; ++k) {
-      c[k] = -l1[k];
-      c[m + k] = -l2[k];
-      c[2 * m + k] = 1.0 / d[k];
-      c[3 * m + k] = -u1[k] / d[k];
-      c[4 * m + k] = -u2[k] / d[k];
-    }
-    for (int q = 0; q < 4; ++q) spk[t][q].assign(m, 0.0);
-    if (!(t & 1)) {  // couplings to the previous chunk's last two values
-      spk[t][0][0] = a;
-      spk[t][1][0] = -4.0 * a; spk[t][1][1] = a;
-    }
-    if (!(t & 2)) {  // couplings to the next chunk's first two values
-      spk[t][2][m - 2] = a; spk[t][2][m - 1] = -4.0 * a;
-      spk[t][3][m - 1] = a;
-    }
-    for (int q = 0; q < 4; ++q) {
-      block_solve(m, l1, l2, d, u1, u2, spk[t][q]);
-      for (int k = 0; k < m; ++k) c[static_cast<size_t>(5 + q) * m + k] = spk[t][q][k];
-    }
-  }
-  const int rows[4] = {0, 1, m - 2, m - 1};
-  const int N4 = 4 * P;
-  std::vector<double> R(static_cast<size_t>(N4) * N4, 0.0);
-  for (int i = 0; i < N4; ++i) R[static_cast<size_t>(i) * N4 + i] = 1.0;
-  for (int p = 0; p < P; ++p) {
-    const int t = (p == 0 ? 1 : 0) | (p == P - 1 ? 2 : 0);
-    for (int r = 0; r < 4; ++r) {
-      const size_t row = static_cast<size_t>(4 * p + r) * N4;
-      if (p > 0) {
-        R[row + 4 * (p - 1) + 2] += spk[t][0][rows[r]];
-        R[row + 4 * (p - 1) + 3] += spk[t][1][rows[r]];
-      }
-      if (p + 1 < P) {
-        R[row + 4 * (p + 1) + 0] += spk[t][2][rows[r]];
-        R[row + 4 * (p + 1) + 1] += spk[t][3][rows[r]];
-      }
-    }
-  }
-  if (!invert(N4, R, K)) return set_error(CS_EINVAL, "Cahn-Hilliard chunk system is singular");
-  return CS_OK;
+// The states entering every chunk of every line: blocks of 8 lines x P chunks.
+template <bool NF>
+__global__ void __launch_bounds__(8 * pn::kMaxChunks)
+    k_line_states(const double* __restrict__ bnd, double* __restrict__ states, const pn::Par q,
+                              const LineTab lt, int64_t lines, int P) {
+  extern __shared__ __align__(16) uint64_t sm[];
+  const int l = threadIdx.x % 8, p = threadIdx.x / 8;
+  const int64_t line = static_cast<int64_t>(blockIdx.x) * 8 + l;
+  double ends[4] = {0.0, 0.0, 0.0, 0.0}, st[4];
+  if (line < lines)
+    for (int j = 0; j < 4; ++j) ends[j] = bnd[(4 * static_cast<int64_t>(p) + j) * lines + line];
+  reduce_states<NF>(q, lt.mats, P, p, reinterpret_cast<double2*>(sm) + l * P, ends, st);
+  if (line < lines)
+    for (int j = 0; j < 4; ++j) states[(4 * static_cast<int64_t>(p) + j) * lines + line] = st[j];
 }
 
-int build_tables(int64_t n, int P, double a, bool noflux, std::vector<double>& coef, std::vector<double>& K) {
-  return noflux ? build_tables_noflux(n, P, a, coef, K) : build_tables_periodic(n, P, a, coef, K);
+template <int MODE, typename T>
+struct AccOut {  // reads W, writes the result of phase 2
+  const uint64_t* p;
+  double* out;
+  T* next;
+  int64_t es;
+  __device__ __forceinline__ void load8(int k, uint64_t (&v)[8]) const {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = p[(k + u) * es];
+  }
+  __device__ __forceinline__ void store8(int k, const uint64_t (&v)[8]) const {
+    if constexpr (MODE == 0) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) out[(k + u) * es] = pn::from_bits(v[u]);
+    } else {
+      T cb[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) cb[u] = next[(k + u) * es];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) next[(k + u) * es] = updated(cb[u], pn::from_bits(v[u]));
+    }
+  }
+};
+
+// MODE 0 writes x (FP64) to out; MODE 1 adds it to Cbar in next.
+template <int MODE, typename T>
+__global__ void __launch_bounds__(kSolveThreads)
+    k_line_correct(uint64_t* __restrict__ G, const double* __restrict__ states, const int* __restrict__ scale,
+                   const pn::Par q, const LineTab lt, int64_t lines, int p0, int Pl, int m, int64_t line_stride,
+                   int64_t elem_stride, double* __restrict__ out, T* __restrict__ next) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= lines * Pl) return;
+  const int64_t line = t % lines, pl = t / lines;
+  const int64_t at = line * line_stride + pl * m * elem_stride;
+  AccOut<MODE, T> s{G + at, MODE == 0 ? out + at : nullptr, MODE == 1 ? next + at : nullptr, elem_stride};
+  double st[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) st[j] = states[(4 * (p0 + pl) + j) * lines + line];
+  correct_chunk(q, TabGlobal(lt), s, m, scale[pl * lines + line], st);
 }
 
 // Valid partition: P divides n, chunks of at least 16 points in whole register batches.
@@ -1066,11 +1037,13 @@ bool valid_chunks(int64_t n, int P) {
   return P >= 1 && P <= 64 && n % P == 0 && (n / P) >= 16 && (n / P) % kU == 0;
 }
 
+// Chunks of at least 16 points up to 32 chunks a line, of at least 32 beyond: the threads of a line
+// are its chunks, and the scan over them costs what a few points do.  Rows + columns on GB300: 512^2
+// 34 us with 32 chunks (39 with 16), 1024^2 48 us with 32 (54 with 16, 56 with 64), 2048^2 114 us with
+// 64 (130 with 32), 4096^2 384 us with 64 (526 with 32).
 int default_chunks(int64_t n) {
-  // enough independent (line, chunk) threads to fill the GPU, while the chunk-end system
-  // (16 P^2 / n FP64 operations per point) stays at most 4 per point
   int P = 1;
-  while (n * P < 65536 && valid_chunks(n, 2 * P) && 16.0 * (2 * P) * (2 * P) / n <= 4.0) P *= 2;
+  while (valid_chunks(n, 2 * P) && n / (2 * P) >= (P < 32 ? 16 : 32)) P *= 2;
   return P;
 }
 
@@ -1107,34 +1080,175 @@ int launch_rhs(CHPlan* p, bool with_rhs, double* partials, cudaStream_t s) {
   return CS_OK;
 }
 
-template <typename T, bool NF>
-void launch_solves(CHPlan* p, cudaStream_t s) {
-  const int64_t n = p->n;
-  const unsigned sgrid = static_cast<unsigned>((n * p->P + kSolveThreads - 1) / kSolveThreads);
-  const size_t ksmem = NF ? 0 : static_cast<size_t>(16) * p->P * sizeof(double);
-  // x-sweep: lines are rows (line stride n, element stride 1)
-  k_solve_local<double, true, NF><<<sgrid, kSolveThreads, 0, s>>>(p->A, p->B, p->bnd, p->coef, n, p->P,
-                                                                  p->m, n, 1);
-  k_solve_correct<0, T, true, NF><<<sgrid, kSolveThreads, ksmem, s>>>(p->B, p->bnd, p->coef, p->K, n, p->P,
-                                                                      p->m, n, 1, p->A, nullptr, nullptr, nullptr);
-  // y-sweep: lines are columns (line stride 1, element stride n), update fused
-  k_solve_local<double, false, NF><<<sgrid, kSolveThreads, 0, s>>>(p->A, p->B, p->bnd, p->coef, n, p->P,
-                                                                   p->m, 1, n);
-  k_solve_correct<1, T, false, NF><<<sgrid, kSolveThreads, ksmem, s>>>(
-      p->B, p->bnd, p->coef, p->K, n, p->P, p->m, 1, n, nullptr,
-      static_cast<const T*>(p->field[p->icur]), static_cast<const T*>(p->field[p->iprev]),
-      static_cast<T*>(p->field[p->inext]));
+LineTab line_tab(const Lines& L) {
+  const pn::TabRow* tab = reinterpret_cast<const pn::TabRow*>(L.tables + static_cast<size_t>(8) * L.P);
+  return {tab, reinterpret_cast<const uint64_t*>(tab + L.m), L.tables};
+}
+// scratch of the global-memory kernels for `lines` lines: end values, states, scale marks
+size_t scratch_doubles(int64_t lines, int P) { return static_cast<size_t>(8) * P * lines + (static_cast<size_t>(P) * lines + 1) / 2; }
+double* line_ends(const Lines& L) { return L.scratch; }
+double* line_states(const Lines& L, int64_t lines) { return L.scratch + static_cast<size_t>(4) * L.P * lines; }
+int* line_scale(const Lines& L, int64_t lines) { return reinterpret_cast<int*>(L.scratch + static_cast<size_t>(8) * L.P * lines); }
+
+void free_lines(Lines* L) {
+  cudaFree(L->tables);
+  cudaFree(L->scratch);
+  L->tables = L->scratch = nullptr;
+}
+
+// Builds the solver for lines of n points in P chunks; scratch_lines > 0 also allocates the scratch.
+int make_lines(int64_t n, int P, double a, bool noflux, int64_t scratch_lines, Lines* L) {
+  std::vector<pn::TabRow> tab;
+  std::vector<uint64_t> base;
+  std::vector<double> mats;
+  L->tables = L->scratch = nullptr;
+  L->P = P;
+  L->m = static_cast<int>(n / P);
+  if (!pn::build(n, P, a, noflux, L->par, tab, base, mats))
+    return set_error(CS_EINVAL, "Cahn-Hilliard line coefficient a = %g is outside the solver's range", a);
+  const size_t nm = mats.size(), nt = 4 * tab.size(), nb = base.size();
+  std::vector<double> all(nm + nt + nb);
+  memcpy(all.data(), mats.data(), nm * 8);
+  memcpy(all.data() + nm, tab.data(), nt * 8);
+  memcpy(all.data() + nm + nt, base.data(), nb * 8);
+  cudaError_t e = cudaMalloc(&L->tables, all.size() * 8);
+  if (e == cudaSuccess && scratch_lines > 0) e = cudaMalloc(&L->scratch, scratch_doubles(scratch_lines, P) * 8);
+  if (e == cudaSuccess) e = cudaMemcpy(L->tables, all.data(), all.size() * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) return CS_OK;
+  free_lines(L);
+  return e == cudaErrorMemoryAllocation ? set_error(CS_ENOMEM, "Cahn-Hilliard line tables: %s", cudaGetErrorString(e))
+                                        : cuda_error(e, "Cahn-Hilliard line tables");
+}
+
+// Shapes of the shared-memory kernels.  Blocks take at most kLineSmem bytes where they can, so that
+// three or more share an SM and one's loads and stores run under the others' arithmetic.
+constexpr size_t kLineSmem = 75 * 1024, kLineSmemMax = 220 * 1024;
+
+// Rows per block (a row takes P (m + 2) words and the scan 2 P), 0 when a row does not fit; one or two
+// warps per block.
+size_t rows_smem(int P, int m, int k) { return static_cast<size_t>(k) * P * (8 * (m + 2) + 16) + kTabBytes * m; }
+int rows_per_block(int64_t rows, int P, int m) {
+  int k = 1;
+  while (k * P < 32 && k < 32) k *= 2;
+  while (k > 1 && (rows % k != 0 || rows_smem(P, m, k) > kLineSmem)) k /= 2;
+  return rows_smem(P, m, k) <= kLineSmemMax ? k : 0;
+}
+
+// Columns per cluster and blocks per cluster, {0, 0} when they do not fit: as many blocks as divide
+// the chunks (eight at most), sixteen columns when that fits kLineSmem, else eight.
+struct ColShape { int nc, cs; };
+size_t cols_smem(int P, int m, ColShape s) {
+  return static_cast<size_t>(P / s.cs) * s.nc * (8 * (m + 1) + 16 + 32) + kTabBytes * m;
+}
+ColShape cols_shape(int P, int m) {
+  int cs = 8;
+  while (P % cs != 0) cs /= 2;
+  const ColShape a{16, cs}, b{8, cs};
+  auto fits = [&](ColShape s, size_t most) { return cols_smem(P, m, s) <= most && s.nc * (P / s.cs) <= 256; };
+  if (fits(a, kLineSmem)) return a;
+  if (fits(b, kLineSmemMax)) return b;
+  return {0, 0};
+}
+
+// The states of `lines` lines from the end values of all their chunks, into the scratch.
+void launch_states(const Lines& L, bool noflux, int64_t lines, const double* ends, cudaStream_t s) {
+  const unsigned grid = static_cast<unsigned>((lines + 7) / 8);
+  const size_t smem = static_cast<size_t>(8) * L.P * sizeof(double2);
+  if (noflux) k_line_states<true><<<grid, 8 * L.P, smem, s>>>(ends, line_states(L, lines), L.par, line_tab(L), lines, L.P);
+  else k_line_states<false><<<grid, 8 * L.P, smem, s>>>(ends, line_states(L, lines), L.par, line_tab(L), lines, L.P);
+}
+
+// Solves along the rows of `rows` x n values (out may equal in).  B: rows x n scratch, used only when a
+// row does not fit in shared memory.
+int launch_rows(const Lines& L, bool noflux, int64_t rows, const double* in, double* out, double* B, cudaStream_t s) {
+  const int P = L.P, m = L.m;
+  const int64_t n = static_cast<int64_t>(P) * m;
+  const LineTab lt = line_tab(L);
+  if (const int k = rows_per_block(rows, P, m)) {
+    const int vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
+    const unsigned grid = static_cast<unsigned>(rows / k);
+    const size_t smem = rows_smem(P, m, k);
+    if (noflux) k_line_rows<true><<<grid, k * P, smem, s>>>(in, out, L.par, lt, P, m, vec);
+    else k_line_rows<false><<<grid, k * P, smem, s>>>(in, out, L.par, lt, P, m, vec);
+    CS_CUDA_TRY(cudaGetLastError());
+    count_launches(1);
+    return CS_OK;
+  }
+  const unsigned grid = static_cast<unsigned>((rows * P + kSolveThreads - 1) / kSolveThreads);
+  k_line_local<<<grid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(B), line_ends(L), line_scale(L, rows), L.par,
+                                              rows, P, m, n, 1);
+  launch_states(L, noflux, rows, line_ends(L), s);
+  k_line_correct<0, double><<<grid, kSolveThreads, 0, s>>>(reinterpret_cast<uint64_t*>(B), line_states(L, rows),
+                                                           line_scale(L, rows), L.par, lt, rows, 0, P, m, n, 1, out,
+                                                           static_cast<double*>(nullptr));
+  CS_CUDA_TRY(cudaGetLastError());
+  count_launches(3);
+  return CS_OK;
+}
+
+// Solves along the columns of the n x n grid and adds the result to Cbar in next.
+template <typename T>
+int launch_cols(const Lines& L, bool noflux, const double* in, T* next, double* B, cudaStream_t s) {
+  const int P = L.P, m = L.m;
+  const int64_t n = static_cast<int64_t>(P) * m;
+  const LineTab lt = line_tab(L);
+  const ColShape sh = cols_shape(P, m);
+  if (sh.nc) {
+    const int vec = (reinterpret_cast<uintptr_t>(next) & (2 * sizeof(T) - 1)) == 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {static_cast<unsigned>(sh.cs), 1, 1};
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(static_cast<unsigned>(n / sh.nc * sh.cs));
+    cfg.blockDim = dim3(static_cast<unsigned>(sh.nc * (P / sh.cs)));
+    cfg.dynamicSmemBytes = cols_smem(P, m, sh);
+    cfg.stream = s;
+    auto kern = noflux ? (sh.nc == 16 ? k_line_cols<16, T, true> : k_line_cols<8, T, true>)
+                       : (sh.nc == 16 ? k_line_cols<16, T, false> : k_line_cols<8, T, false>);
+    CS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, in, next, n, L.par, lt, P, m, vec));
+    count_launches(1);
+    return CS_OK;
+  }
+  const unsigned grid = static_cast<unsigned>((n * P + kSolveThreads - 1) / kSolveThreads);
+  k_line_local<<<grid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(B), line_ends(L), line_scale(L, n), L.par, n, P,
+                                              m, 1, n);
+  launch_states(L, noflux, n, line_ends(L), s);
+  k_line_correct<1, T><<<grid, kSolveThreads, 0, s>>>(reinterpret_cast<uint64_t*>(B), line_states(L, n), line_scale(L, n),
+                                                      L.par, lt, n, 0, P, m, 1, n, nullptr, next);
+  CS_CUDA_TRY(cudaGetLastError());
+  count_launches(3);
+  return CS_OK;
+}
+
+// The shared-memory kernels' size limit, set before any launch or capture.
+int set_line_attrs() {
+  const int bytes = static_cast<int>(kLineSmemMax);
+  const void* kerns[] = {
+      reinterpret_cast<const void*>(k_line_rows<false>), reinterpret_cast<const void*>(k_line_rows<true>),
+#define CS_LINE_COLS(T, NF)                                   \
+  reinterpret_cast<const void*>(k_line_cols<8, T, NF>), reinterpret_cast<const void*>(k_line_cols<16, T, NF>)
+      CS_LINE_COLS(double, false), CS_LINE_COLS(double, true), CS_LINE_COLS(float, false), CS_LINE_COLS(float, true)
+#undef CS_LINE_COLS
+  };
+  for (const void* k : kerns) CS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  return CS_OK;
+}
+
+// Whether a full-grid plan needs the global-memory kernels' scratch.
+bool needs_scratch(int64_t n, int P) {
+  const int m = static_cast<int>(n / P);
+  return !rows_per_block(n, P, m) || !cols_shape(P, m).nc;
 }
 
 template <typename T>
 int launch_step(CHPlan* p, double* partials, cudaStream_t s) {
   int rc = launch_rhs<T>(p, true, partials, s);
   if (rc != CS_OK) return rc;
-  if (p->noflux) launch_solves<T, true>(p, s);
-  else launch_solves<T, false>(p, s);
-  CS_CUDA_TRY(cudaGetLastError());
-  count_launches(4);
-  return CS_OK;
+  rc = launch_rows(p->lines, p->noflux != 0, p->n, p->A, p->A, p->B, s);
+  if (rc != CS_OK) return rc;
+  return launch_cols<T>(p->lines, p->noflux != 0, p->A, static_cast<T*>(p->field[p->inext]), p->B, s);
 }
 
 void rotate(CHPlan* p) {
@@ -1158,7 +1272,8 @@ int reduce_current(CHPlan* p, double* out2, cudaStream_t s) {
 void free_plan(CHPlan* p) {
   if (!p) return;
   drop_graphs(p);
-  cudaFree(p->A); cudaFree(p->B); cudaFree(p->bnd); cudaFree(p->coef); cudaFree(p->K);
+  free_lines(&p->lines);
+  cudaFree(p->A); cudaFree(p->B);
   cudaFree(p->partials); cudaFree(p->inv); cudaFree(p->diag);
   delete p;
 }
@@ -1209,25 +1324,20 @@ int ch_create(CHPlan** out, const cs_ch_desc* d, void* prev, void* cur, void* ne
   p->field[0] = prev; p->field[1] = cur; p->field[2] = next;
   p->iprev = 0; p->icur = 1; p->inext = 2;
   p->rhs_blocks = static_cast<int>((d->n / kTX) * (d->n / kTY));
-  std::vector<double> coef, K;
-  int rc = build_tables(d->n, P, p->a, p->noflux != 0, coef, K);
+  int rc = make_lines(d->n, P, p->a, p->noflux != 0, needs_scratch(d->n, P) ? d->n : 0, &p->lines);
   if (rc != CS_OK) { free_plan(p); return rc; }
   const size_t nn = static_cast<size_t>(d->n) * d->n;
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = cudaMalloc(&p->A, nn * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&p->B, nn * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&p->bnd, static_cast<size_t>(4) * P * d->n * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&p->coef, coef.size() * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&p->K, K.size() * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&p->partials, static_cast<size_t>(2) * p->rhs_blocks * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemcpy(p->coef, coef.data(), coef.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(p->K, K.data(), K.size() * sizeof(double), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     free_plan(p);
     return e == cudaErrorMemoryAllocation ? set_error(CS_ENOMEM, "Cahn-Hilliard workspace: %s", cudaGetErrorString(e))
                                           : cuda_error(e, "Cahn-Hilliard workspace");
   }
   rc = d->storage == CS_F32 ? set_rhs_attr<float>() : set_rhs_attr<double>();  // before any capture
+  if (rc == CS_OK) rc = set_line_attrs();
   if (rc != CS_OK) { free_plan(p); return rc; }
   *out = p;
   return CS_OK;
@@ -1560,24 +1670,14 @@ int ch_fields(CHPlan* p, void** prev, void** cur, int64_t* steps) {
 
 namespace {
 
-// (Re)builds the partition tables and chunk-end buffer for P chunks per line.
+// (Re)builds the line solver for P chunks per line.
 int set_partition(CHPlan* p, int P) {
-  std::vector<double> coef, K;
-  int rc = build_tables(p->n, P, p->a, p->noflux != 0, coef, K);
+  Lines L;
+  int rc = make_lines(p->n, P, p->a, p->noflux != 0, needs_scratch(p->n, P) ? p->n : 0, &L);
   if (rc != CS_OK) return rc;
-  double *bnd = nullptr, *dcoef = nullptr, *dK = nullptr;
-  cudaError_t e = cudaMalloc(&bnd, static_cast<size_t>(4) * P * p->n * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&dcoef, coef.size() * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&dK, K.size() * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemcpy(dcoef, coef.data(), coef.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dK, K.data(), K.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(bnd); cudaFree(dcoef); cudaFree(dK);
-    return cuda_error(e, "Cahn-Hilliard partition tables");
-  }
   drop_graphs(p);
-  cudaFree(p->bnd); cudaFree(p->coef); cudaFree(p->K);
-  p->bnd = bnd; p->coef = dcoef; p->K = dK;
+  free_lines(&p->lines);
+  p->lines = L;
   p->P = P;
   p->m = static_cast<int>(p->n / P);
   return CS_OK;
@@ -1678,10 +1778,8 @@ struct CHBand {
   int noflux;  // CS_CH_NOFLUX: mirrored columns, non-cyclic line solves
   double D, gamma, dt, h, a, alpha;
   int P, m;
-  double* coef;
-  double* K;
-  double* B;         // rows * n scratch (local solutions)
-  double* bnd;       // 4 * P * rows chunk-end values
+  Lines lines;       // scratch for n lines: the band's columns, or its rows
+  double* B;         // rows * n scratch (the local solutions of the columns, or of rows that do not fit in shared memory)
   double* partials;  // 2 per RHS block
   int rhs_blocks;
 };
@@ -1704,7 +1802,8 @@ __global__ void __launch_bounds__(256)
 
 void free_band(CHBand* b) {
   if (!b) return;
-  cudaFree(b->coef); cudaFree(b->K); cudaFree(b->B); cudaFree(b->bnd); cudaFree(b->partials);
+  free_lines(&b->lines);
+  cudaFree(b->B); cudaFree(b->partials);
   delete b;
 }
 }  // namespace
@@ -1744,22 +1843,17 @@ int ch_band_create(CHBand** out, const cs_ch_desc* d, int64_t rows) {
   b->P = P;
   b->m = static_cast<int>(d->n / P);
   b->rhs_blocks = static_cast<int>((d->n / kTX) * (rows / kTY));
-  std::vector<double> coef, K;
-  int rc = build_tables(d->n, P, b->a, b->noflux != 0, coef, K);
+  int rc = make_lines(d->n, P, b->a, b->noflux != 0, d->n, &b->lines);
   if (rc != CS_OK) { free_band(b); return rc; }
-  cudaError_t e = cudaMalloc(&b->coef, coef.size() * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&b->K, K.size() * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&b->B, static_cast<size_t>(rows) * d->n * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&b->bnd, static_cast<size_t>(4) * P * rows * sizeof(double));
+  cudaError_t e = cudaMalloc(&b->B, static_cast<size_t>(rows) * d->n * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&b->partials, static_cast<size_t>(2) * b->rhs_blocks * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemcpy(b->coef, coef.data(), coef.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(b->K, K.data(), K.size() * sizeof(double), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     free_band(b);
     return e == cudaErrorMemoryAllocation ? set_error(CS_ENOMEM, "band workspace: %s", cudaGetErrorString(e))
                                           : cuda_error(e, "band workspace");
   }
   rc = d->storage == CS_F32 ? set_rhs_attr<float>() : set_rhs_attr<double>();
+  if (rc == CS_OK) rc = set_line_attrs();
   if (rc != CS_OK) { free_band(b); return rc; }
   *out = b;
   return CS_OK;
@@ -1792,23 +1886,8 @@ int ch_band_rhs(CHBand* b, const void* prev, const void* cur, double* rhs, doubl
 
 int ch_band_solve(CHBand* b, const double* in, double* out, cudaStream_t s) {
   if (!in || !out) return set_error(CS_EINVAL, "null buffer");
-  const unsigned sgrid = static_cast<unsigned>((b->rows * b->P + kSolveThreads - 1) / kSolveThreads);
-  // rows lines of n points, line stride n, element stride 1 (the kernels' line count is `rows`)
-  if (b->noflux) {
-    k_solve_local<double, true, true><<<sgrid, kSolveThreads, 0, s>>>(in, b->B, b->bnd, b->coef, b->rows, b->P,
-                                                                     b->m, b->n, 1);
-    k_solve_correct<0, double, true, true><<<sgrid, kSolveThreads, 0, s>>>(
-        b->B, b->bnd, b->coef, b->K, b->rows, b->P, b->m, b->n, 1, out, nullptr, nullptr, nullptr);
-  } else {
-    const size_t ksmem = static_cast<size_t>(16) * b->P * sizeof(double);
-    k_solve_local<double, true, false><<<sgrid, kSolveThreads, 0, s>>>(in, b->B, b->bnd, b->coef, b->rows, b->P,
-                                                                      b->m, b->n, 1);
-    k_solve_correct<0, double, true, false><<<sgrid, kSolveThreads, ksmem, s>>>(
-        b->B, b->bnd, b->coef, b->K, b->rows, b->P, b->m, b->n, 1, out, nullptr, nullptr, nullptr);
-  }
-  CS_CUDA_TRY(cudaGetLastError());
-  count_launches(2);
-  return CS_OK;
+  // rows lines of n points
+  return launch_rows(b->lines, b->noflux != 0, b->rows, in, out, b->B, s);
 }
 
 int ch_partition(const cs_ch_desc* d, int32_t* chunks, int32_t* chunk_len) {
@@ -1842,12 +1921,8 @@ int ch_band_ycols_local(CHBand* b, int64_t chunk0, const double* in, double* end
   if (rc != CS_OK) return rc;
   const int Pl = static_cast<int>(b->rows / b->m);
   const unsigned sgrid = static_cast<unsigned>((b->n * Pl + kSolveThreads - 1) / kSolveThreads);
-  if (b->noflux)
-    k_solve_local<double, false, true><<<sgrid, kSolveThreads, 0, s>>>(in, b->B, ends, b->coef, b->n, b->P, b->m, 1,
-                                                                       b->n, static_cast<int>(chunk0), Pl);
-  else
-    k_solve_local<double, false, false><<<sgrid, kSolveThreads, 0, s>>>(in, b->B, ends, b->coef, b->n, b->P, b->m, 1,
-                                                                        b->n, static_cast<int>(chunk0), Pl);
+  k_line_local<<<sgrid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(b->B), ends, line_scale(b->lines, b->n),
+                                               b->lines.par, b->n, Pl, b->m, 1, b->n);
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return CS_OK;
@@ -1859,18 +1934,12 @@ int ch_band_ycols_correct(CHBand* b, int64_t chunk0, const double* ends_all, dou
   if (rc != CS_OK) return rc;
   const int Pl = static_cast<int>(b->rows / b->m);
   const unsigned sgrid = static_cast<unsigned>((b->n * Pl + kSolveThreads - 1) / kSolveThreads);
-  if (b->noflux) {
-    k_solve_correct<0, double, false, true><<<sgrid, kSolveThreads, 0, s>>>(
-        b->B, ends_all, b->coef, b->K, b->n, b->P, b->m, 1, b->n, v, nullptr, nullptr, nullptr,
-        static_cast<int>(chunk0), Pl);
-  } else {
-    const size_t ksmem = static_cast<size_t>(16) * b->P * sizeof(double);
-    k_solve_correct<0, double, false, false><<<sgrid, kSolveThreads, ksmem, s>>>(
-        b->B, ends_all, b->coef, b->K, b->n, b->P, b->m, 1, b->n, v, nullptr, nullptr, nullptr,
-        static_cast<int>(chunk0), Pl);
-  }
+  launch_states(b->lines, b->noflux != 0, b->n, ends_all, s);
+  k_line_correct<0, double><<<sgrid, kSolveThreads, 0, s>>>(
+      reinterpret_cast<uint64_t*>(b->B), line_states(b->lines, b->n), line_scale(b->lines, b->n), b->lines.par,
+      line_tab(b->lines), b->n, static_cast<int>(chunk0), Pl, b->m, 1, b->n, v, static_cast<double*>(nullptr));
   CS_CUDA_TRY(cudaGetLastError());
-  count_launches(1);
+  count_launches(2);
   return CS_OK;
 }
 
@@ -1891,78 +1960,25 @@ int ch_band_update(CHBand* b, const void* prev, const void* cur, const double* v
 
 void ch_band_destroy(CHBand* b) { free_band(b); }
 
-// Host replay of the device line solver (phase 1: chunk LU forward and backward, chunk-end
-// values; phase 2: neighbouring chunk ends from K, spike correction), in the kernels' order of
-// operations, on the tables cs_ch_create builds, for a pseudo-random right-hand side; returns the
-// backward error ||L x - b||_inf / ((1 + 16 a) ||x||_inf) of the result against the line operator
+// Host replay of the device line solver (the kernels' own functions, in their order) on the tables
+// cs_ch_create builds, for a pseudo-random right-hand side; returns the backward error ||L x - b||_inf / ((1 + 16 a) ||x||_inf) of the result against the line operator
 // itself (periodic: circulant (1, -4, 6, -4, 1); no-flux: reflected rows at the ends).
 int ch_solver_check(int64_t n, int P, double a, bool noflux, double* residual) {
   if (!residual) return set_error(CS_EINVAL, "null residual pointer");
   if (n < 16 || n > 65536 || !valid_chunks(n, P)) return set_error(CS_EINVAL, "invalid line length / chunk count");
   if (!(a >= 0.0) || !std::isfinite(a)) return set_error(CS_EINVAL, "a must be finite and >= 0");
-  std::vector<double> coef, K;
-  int rc = build_tables(n, P, a, noflux, coef, K);
-  if (rc != CS_OK) return rc;
-  const int m = static_cast<int>(n / P);
-  std::vector<double> b(n), g(n), x(n), ends(static_cast<size_t>(4) * P);
+  pn::Par q;
+  std::vector<pn::TabRow> tab;
+  std::vector<uint64_t> base;
+  std::vector<double> mats;
+  if (!pn::build(n, P, a, noflux, q, tab, base, mats)) return set_error(CS_EINVAL, "a = %g is outside the solver's range", a);
+  std::vector<double> b(n), x(n);
   uint64_t st = 0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(n * 131 + P);
   for (int64_t i = 0; i < n; ++i) {  // xorshift64*: values in [-1, 1)
     st ^= st >> 12; st ^= st << 25; st ^= st >> 27;
     b[i] = static_cast<double>((st * 0x2545F4914F6CDD1Dull) >> 11) * 0x1p-52 - 1.0;
   }
-  auto tab = [&](int p) { return coef.data() + (noflux ? static_cast<size_t>(9) * m * chunk_type(p, P) : 0); };
-  for (int p = 0; p < P; ++p) {  // phase 1
-    const double* c = tab(p);
-    double y1 = 0.0, y2 = 0.0;
-    for (int k = 0; k < m; ++k) {
-      const double y = fma(c[k], y1, fma(c[m + k], y2, b[p * m + k]));
-      g[p * m + k] = y;
-      y2 = y1;
-      y1 = y;
-    }
-    double g1 = 0.0, g2 = 0.0;
-    for (int k = m - 1; k >= 0; --k) {
-      const double v = fma(c[3 * m + k], g1, fma(c[4 * m + k], g2, g[p * m + k] * c[2 * m + k]));
-      g[p * m + k] = v;
-      g2 = g1;
-      g1 = v;
-    }
-    ends[4 * p] = g[p * m];
-    ends[4 * p + 1] = g[p * m + 1];
-    ends[4 * p + 2] = g[p * m + m - 2];
-    ends[4 * p + 3] = g[p * m + m - 1];
-  }
-  const int64_t N4 = 4 * static_cast<int64_t>(P);
-  for (int p = 0; p < P; ++p) {  // phase 2
-    double t0 = 0.0, t1 = 0.0, h0 = 0.0, h1 = 0.0;
-    for (int q = 0; q < P; ++q) {
-      const double* e = ends.data() + 4 * q;
-      if (noflux) {
-        if (p > 0) {
-          const double* r2 = K.data() + (4 * static_cast<int64_t>(p - 1) + 2) * N4 + 4 * q;
-          const double* r3 = r2 + N4;
-          t0 = fma(r2[0], e[0], fma(r2[1], e[1], fma(r2[2], e[2], fma(r2[3], e[3], t0))));
-          t1 = fma(r3[0], e[0], fma(r3[1], e[1], fma(r3[2], e[2], fma(r3[3], e[3], t1))));
-        }
-        if (p + 1 < P) {
-          const double* r0 = K.data() + 4 * static_cast<int64_t>(p + 1) * N4 + 4 * q;
-          const double* r1 = r0 + N4;
-          h0 = fma(r0[0], e[0], fma(r0[1], e[1], fma(r0[2], e[2], fma(r0[3], e[3], h0))));
-          h1 = fma(r1[0], e[0], fma(r1[1], e[1], fma(r1[2], e[2], fma(r1[3], e[3], h1))));
-        }
-      } else {
-        const double* Kt = K.data() + ((p + P - 1 - q + P) % P) * 16;
-        const double* Kh = K.data() + ((p + 1 - q + P) % P) * 16;
-        t0 = fma(Kt[8], e[0], fma(Kt[9], e[1], fma(Kt[10], e[2], fma(Kt[11], e[3], t0))));
-        t1 = fma(Kt[12], e[0], fma(Kt[13], e[1], fma(Kt[14], e[2], fma(Kt[15], e[3], t1))));
-        h0 = fma(Kh[0], e[0], fma(Kh[1], e[1], fma(Kh[2], e[2], fma(Kh[3], e[3], h0))));
-        h1 = fma(Kh[4], e[0], fma(Kh[5], e[1], fma(Kh[6], e[2], fma(Kh[7], e[3], h1))));
-      }
-    }
-    const double* c = tab(p);
-    for (int k = 0; k < m; ++k)
-      x[p * m + k] = fma(-c[5 * m + k], t0, fma(-c[6 * m + k], t1, fma(-c[7 * m + k], h0, fma(-c[8 * m + k], h1, g[p * m + k]))));
-  }
+  pn::solve_host(q, tab, base, mats, n, P, noflux, b.data(), x.data());
   double rmax = 0.0, xmax = 0.0;
   auto at = [&](int64_t i) {  // periodic wrap or even reflection
     if (!noflux) return x[(i % n + n) % n];

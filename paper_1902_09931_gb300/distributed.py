@@ -10,7 +10,7 @@ ranks (Sec. 6.2, MPI).  Here:
 * Cahn-Hilliard ADI (Sec. 5.1): the right-hand side needs a 2-row halo of C^n and C^{n-1}; the
   x-line solves are local to a row band.  The y lines are cut into the partitioned solver's
   chunks; when the bands are whole numbers of chunks each rank solves its own chunks and the ranks
-  all-gather only the chunks' end values (4 per column and chunk) for the spike correction;
+  all-gather only the chunks' end values (4 per column and chunk) for the correction;
   otherwise the y-line solves run after an all-to-all transpose that gives every rank a band of
   columns, and a second transpose brings the result back.  Mass and energy are sums of per-rank
   FP64 partials (an allreduce).
@@ -340,10 +340,10 @@ class DeviceCHBand:
     of `group`, one band per rank, computed by this library's band entry points (cs_ch_band_*):
     halo exchange of C^n and C^{n-1} (2 rows, in place in padded buffers), the band's right-hand
     side, the x line solves, the y line solves and the update.  The y lines run in one of two ways:
-      * "chunks" (whenever the spike method's chunks of a line, cs_ch_partition, split evenly over
+      * "chunks" (whenever the partitioned solver's chunks of a line, cs_ch_partition, split evenly over
         the ranks: then every band is a whole number of chunks of every column): each rank solves
         its chunks locally (cs_ch_band_ycols_local), the ranks all-gather the chunks' end values (4
-        per column and chunk: 4 * chunks * n values in all), and each applies the spike correction
+        per column and chunk: 4 * chunks * n values in all), and each applies the correction
         to its own chunks (cs_ch_band_ycols_correct); the field never moves between ranks;
       * "transposes" (otherwise): an all-to-all transpose gives each rank a band of columns, solved
         as rows, and a second transpose brings the result back.
