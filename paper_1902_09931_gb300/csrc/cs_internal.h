@@ -44,6 +44,8 @@ struct Stencil2DConfig {
   float* d_weights_f; // FP32 copy
   int dd_ok;          // weights fit the double-float path (FP64 storage)
   int use_tma;        // tile choice 2: TMA-pipelined persistent sweep (aligned buffers)
+  int auto_shape;     // no choice made by the caller or the autotuner: the sweep picks by size
+  int64_t cells;      // grid points of the description (a streamed plan's band slots keep it)
   mutable CUtensorMap tmap;      // tensor map of the last input pointer (rebuilt on change)
   mutable const void* tmap_in;
   int ix_ok;          // weights are c * small integers: exact digit path (FP64 storage)

@@ -61,6 +61,8 @@ int stencil2d_prepare(Stencil2DConfig* cfg) {
   cfg->tmap_in = nullptr;
   if (cfg->tile_rows != 32 && cfg->tile_rows != 64) cfg->tile_rows = 64;
   cfg->use_tma = 1;
+  cfg->auto_shape = 1;
+  cfg->cells = cfg->nx * cfg->ny;
   const int W = cfg->left + cfg->right + 1, H = cfg->top + cfg->bottom + 1;
   if (cfg->fn != CS_FN_NONE) {
     int rc = map_function(cfg);
@@ -205,6 +207,7 @@ int stencil2d_check(const Stencil2DConfig* cfg, cudaStream_t s) {
 int stencil2d_num_tile_choices() { return 3; }
 
 int stencil2d_set_tile_choice(Stencil2DConfig* cfg, int choice) {
+  cfg->auto_shape = 0;
   cfg->use_tma = choice == 2;
   cfg->tile_rows = choice == 0 ? 32 : 64;
   return CS_OK;

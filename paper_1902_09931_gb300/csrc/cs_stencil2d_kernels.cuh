@@ -148,36 +148,49 @@ __device__ __forceinline__ void load_tile(T* s, const T* __restrict__ in, int64_
     __syncthreads();
     return;
   }
+  // Any other tile.  Where rows are 16-byte aligned (nx a multiple of V; the tile's columns start at
+  // one) a 16-byte chunk lies inside the grid or outside it as a whole, so it wraps as a chunk; else
+  // element by element, without the wraps where the tile lies inside the grid.
   const bool one_wrap = nx >= cols && ny >= rows;  // tile halo reaches at most one period out
-  for (int idx = threadIdx.x; idx < total; idx += kThreads) {
-    const int r = idx / nch;
-    const int ch = idx - r * nch;
-    T* dst = s + r * cols + ch * V;
-    int64_t gy = y0 - top + r;
-    if (gy < 0 || gy >= ny) {
-      if (!periodic) {
-#pragma unroll
-        for (int e = 0; e < V; ++e) dst[e] = T(0);
-        continue;
-      }
-      gy = one_wrap ? (gy < 0 ? gy + ny : gy - ny) : wrap_idx(gy, ny);
-    }
-    const T* row = in + gy * nx;
-    const int64_t gx0 = x0 - LA + static_cast<int64_t>(ch) * V;
-    if (vec_ok && gx0 >= 0 && gx0 + V <= nx) {
-      cp_async16(dst, row + gx0);
-    } else {
-#pragma unroll
-      for (int e = 0; e < V; ++e) {
-        int64_t gx = gx0 + e;
-        if (gx < 0 || gx >= nx) {
-          if (!periodic) {
-            dst[e] = T(0);
-            continue;
-          }
-          gx = one_wrap ? (gx < 0 ? gx + nx : gx - nx) : wrap_idx(gx, nx);
+  auto wrapped = [&](int64_t k, int64_t n) { return one_wrap ? (k < 0 ? k + n : (k >= n ? k - n : k)) : wrap_idx(k, n); };
+  if (vec_ok) {
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < total; idx += kThreads) {
+      const int r = idx / nch, ch = idx - r * nch;
+      int64_t gy = gy0 + r, gx = gx0 + static_cast<int64_t>(ch) * V;
+      T* dst = s + r * cols + ch * V;
+      const bool inside = gy >= 0 && gy < ny && gx >= 0 && gx < nx;
+      if (inside || periodic) {
+        if (!inside) {
+          gy = wrapped(gy, ny);
+          gx = wrapped(gx, nx);
         }
-        cp_async_elem(dst + e, row + gx);
+        cp_async16(dst, in + gy * nx + gx);
+      } else {
+        *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  } else if (gy0 >= 0 && gy0 + rows <= ny && gx0 >= 0 && gx0 + cols <= nx) {
+    const T* src = in + gy0 * nx + gx0;
+#pragma unroll 6
+    for (int idx = threadIdx.x; idx < rows * cols; idx += kThreads) {
+      const int r = idx / cols, c = idx - r * cols;
+      cp_async_elem(s + idx, src + static_cast<int64_t>(r) * nx + c);
+    }
+  } else {
+#pragma unroll 2
+    for (int idx = threadIdx.x; idx < rows * cols; idx += kThreads) {
+      const int r = idx / cols, c = idx - r * cols;
+      int64_t gy = gy0 + r, gx = gx0 + c;
+      const bool inside = gy >= 0 && gy < ny && gx >= 0 && gx < nx;
+      if (inside || periodic) {
+        if (!inside) {
+          gy = wrapped(gy, ny);
+          gx = wrapped(gx, nx);
+        }
+        cp_async_elem(s + idx, in + gy * nx + gx);
+      } else {
+        s[idx] = T(0);
       }
     }
   }
@@ -899,7 +912,9 @@ int launch_group_t(const Stencil2DConfig* const* cfgs, const void* const* ins, v
                    int count, cudaStream_t st) {
   GroupTable<T> tab;
   memset(&tab, 0, sizeof tab);
-  const int variant = cfgs[0]->variant, TY = cfgs[0]->tile_rows;
+  // FP32 storage gives the same bits with either tile height: 32 rows, so that a batch of small grids
+  // spreads over twice the CTAs
+  const int variant = cfgs[0]->variant, TY = sizeof(T) == 4 ? 32 : cfgs[0]->tile_rows;
   const SpecDesc& sd = kSpecs[variant];
   const int nt = (sd.L + sd.R + 1) * (sd.T + sd.B + 1);
   bool digits = sizeof(T) == 8 && !sd.xform;
@@ -1519,10 +1534,34 @@ static_assert(kNumSpecs == 14, "update dispatch_spec");
 
 int make_tensor_map(const Stencil2DConfig* cfg, const void* in, int elem_bytes, int cols, int rows);
 
+// The tile shape a sweep runs with: the plan's own where the caller or the autotuner chose one, else
+// by size (times on GB300, back to back, us; the same bits for FP32 storage whatever the shape, and for
+// FP64 storage between 64-row tiles and TMA):
+//   FP64 storage on the digit or double-float path: tiles of 32 rows up to 2^22.5 points, where more
+//   CTAs hide each other's load and reduction phases (9-point Laplacian, 256^2 3.8 against 5.4 with 64
+//   rows and 5.7 with TMA; 2048^2 18.2 / 19.8 / 20.9; 3072^2 34.9 / 34.6 / 38.5), 64 rows beyond
+//   (4096^2 57.6 / 54.6 / 61.4; 8192^2 biharmonic 230 / 203 / 240), and 32 rows for rows that are not
+//   16-byte aligned (4097^2 69.0 / 77.2);
+//   FP32 storage: 32 rows (512^2 2.7 / 3.5 / 4.0; 4096^2 23.7 / 24.1 / 24.3; 8192^2 84.5 / 84.0 /
+//   94.8; 4097^2 32.1 / 38.3), except TMA for non-periodic stencils that reach sideways on 2^20 to
+//   2^23 points (2048^2 7.6 / 7.4 / 7.1).
+struct TileShape { int rows; bool tma; };
+template <typename T> TileShape tile_shape(const Stencil2DConfig* cfg) {
+  if (!cfg->auto_shape || cfg->variant < 0) return {cfg->tile_rows, cfg->use_tma != 0};
+  const int64_t cells = cfg->cells;
+  if (sizeof(T) == 8) {
+    if (cfg->fp64_mode != CS_FP64_AUTO || !(cfg->ix_ok || cfg->dd_ok)) return {cfg->tile_rows, cfg->use_tma != 0};
+    return {cells <= 5931641 || cfg->nx % 2 != 0 ? 32 : 64, false};
+  }
+  const bool tma = cfg->bc != CS_BC_PERIODIC && cfg->left + cfg->right > 0 && cells > (1 << 20) && cells <= (1 << 23);
+  return {tma ? 64 : 32, tma};
+}
+
 template <typename T>
 int launch_stencil2d_t(const Stencil2DConfig* cfg, const void* vin, void* vout, cudaStream_t st) {
   const T* in = static_cast<const T*>(vin);
   T* out = static_cast<T*>(vout);
+  const TileShape shape = tile_shape<T>(cfg);
   const int periodic = cfg->bc == CS_BC_PERIODIC;
   const int vec_ok = (cfg->nx % Vec<T>::n == 0) && (reinterpret_cast<uintptr_t>(in) % 16 == 0);
   if (cfg->variant >= 0) {
@@ -1530,7 +1569,7 @@ int launch_stencil2d_t(const Stencil2DConfig* cfg, const void* vin, void* vout, 
     const SpecDesc& sd = kSpecs[cfg->variant];
     const int nt = (sd.L + sd.R + 1) * (sd.T + sd.B + 1);
     for (int i = 0; i < 32; ++i) taps.w[i] = i < nt ? static_cast<T>(cfg->weights[i]) : T(0);
-    if (cfg->use_tma && vec_ok && cfg->nx < (int64_t(1) << 31) && cfg->ny < (int64_t(1) << 31)) {
+    if (shape.tma && vec_ok && cfg->nx < (int64_t(1) << 31) && cfg->ny < (int64_t(1) << 31)) {
       constexpr int V = Vec<T>::n;
       const int LA = (sd.L + V - 1) / V * V, RA = (sd.R + V - 1) / V * V;
       const int cols = LA + tile_x<T>() + RA, rows = 64 + sd.T + sd.B;
@@ -1577,7 +1616,7 @@ int launch_stencil2d_t(const Stencil2DConfig* cfg, const void* vin, void* vout, 
         it.c15 = -1.5 * it.c;
         it.inv_hi = static_cast<float>(1.0 / cfg->ix_c);
         it.inv_lo = static_cast<float>(1.0 / cfg->ix_c - static_cast<double>(it.inv_hi));
-        if (cfg->tile_rows == 32)
+        if (shape.rows == 32)
           return dispatch_ix<32>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, it, cfg, st);
         return dispatch_ix<64>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, it, cfg, st);
       }
@@ -1588,12 +1627,12 @@ int launch_stencil2d_t(const Stencil2DConfig* cfg, const void* vin, void* vout, 
           dt.hi[i] = static_cast<float>(w);
           dt.lo[i] = static_cast<float>(w - static_cast<double>(dt.hi[i]));
         }
-        if (cfg->tile_rows == 32)
+        if (shape.rows == 32)
           return dispatch_dd<32>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, dt, st);
         return dispatch_dd<64>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, dt, st);
       }
     }
-    if (cfg->tile_rows == 32)
+    if (shape.rows == 32)
       return dispatch_spec<T, 32>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, st);
     return dispatch_spec<T, 64>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, st);
   }
@@ -1601,7 +1640,7 @@ int launch_stencil2d_t(const Stencil2DConfig* cfg, const void* vin, void* vout, 
   if constexpr (sizeof(T) == 8) d_w = reinterpret_cast<const T*>(cfg->d_weights);
   else d_w = reinterpret_cast<const T*>(cfg->d_weights_f);
   const int xform = cfg->fn == CS_FN_CH_NONLIN_LAP, epi = cfg->fn == CS_FN_CUBIC_MINUS_LAP;
-  if (cfg->tile_rows == 32)
+  if (shape.rows == 32)
     return launch_generic<T, 32>(in, out, cfg, d_w, periodic, vec_ok, xform, epi, st);
   return launch_generic<T, 64>(in, out, cfg, d_w, periodic, vec_ok, xform, epi, st);
 }
