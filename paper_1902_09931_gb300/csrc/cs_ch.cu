@@ -634,6 +634,8 @@ struct AccRow {  // words in a row, 16-byte aligned (shared memory)
 #pragma unroll
     for (int u = 0; u < 8; u += 2) *reinterpret_cast<ulonglong2*>(p + k + u) = make_ulonglong2(v[u], v[u + 1]);
   }
+  __device__ __forceinline__ uint64_t get(int k) const { return p[k]; }
+  __device__ __forceinline__ void put(int k, uint64_t v) const { p[k] = v; }
 };
 struct AccStride {  // words es apart (shared or global memory)
   uint64_t* p;
@@ -646,6 +648,8 @@ struct AccStride {  // words es apart (shared or global memory)
 #pragma unroll
     for (int u = 0; u < 8; ++u) p[(k + u) * es] = v[u];
   }
+  __device__ __forceinline__ uint64_t get(int k) const { return p[k * es]; }
+  __device__ __forceinline__ void put(int k, uint64_t v) const { p[k * es] = v; }
 };
 template <int ES>
 struct AccCols {  // ES columns interleaved (shared memory)
@@ -658,6 +662,8 @@ struct AccCols {  // ES columns interleaved (shared memory)
 #pragma unroll
     for (int u = 0; u < 8; ++u) p[(k + u) * ES] = v[u];
   }
+  __device__ __forceinline__ uint64_t get(int k) const { return p[k * ES]; }
+  __device__ __forceinline__ void put(int k, uint64_t v) const { p[k * ES] = v; }
 };
 
 // The states entering chunk p of a line from all its chunks' end values: inclusive scans over the
@@ -784,11 +790,11 @@ struct TabGlobal {
 };
 constexpr int kTabBytes = 40;  // per point of a chunk
 
-// Starts the copy of the tables to shared memory (16-byte aligned, kTabBytes m): rows, then bias terms
-// (m is a multiple of 8).  The caller waits for it with its other copies.
+// Starts the copy of the tables to shared memory (16-byte aligned, kTabBytes m): rows, then bias
+// terms.  The caller waits for it with its other copies.
 __device__ __forceinline__ TabShared stage_tables(uint64_t* to, const LineTab& lt, int m) {
   for (int i = threadIdx.x; i < 2 * m; i += blockDim.x) cp_async16(to + 2 * i, reinterpret_cast<const uint64_t*>(lt.tab) + 2 * i);
-  for (int i = threadIdx.x; i < m / 2; i += blockDim.x) cp_async16(to + 4 * m + 2 * i, lt.base + 2 * i);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) cp_async8(to + 4 * m + i, lt.base + i);
   return {reinterpret_cast<const ulonglong2*>(to), to + 4 * m};
 }
 
@@ -798,30 +804,26 @@ __device__ __forceinline__ void correct_chunk(const pn::Par& q, const Tab& tab, 
                                               const double (&st)[4]) {
   pn::Corr c;
   if (pn::corr_setup(q, ew, st, c)) {
-    for (int k0 = 0; k0 < m; k0 += 8) {
+    auto point = [&](int k, uint64_t w) {
+      uint64_t t[4], b;
+      tab.row(k, t, b);
+      return pn::dbits(pn::from_fixed(pn::corr_point(c, w, t, b), c.eo));
+    };
+    for (int k0 = 0; k0 + 8 <= m; k0 += 8) {
       uint64_t v[8];
       s.load8(k0, v);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        uint64_t t[4], b;
-        tab.row(k0 + u, t, b);
-        v[u] = pn::dbits(pn::from_fixed(pn::corr_point(c, v[u], t, b), c.eo));
-      }
+      for (int u = 0; u < 8; ++u) v[u] = point(k0 + u, v[u]);
       s.store8(k0, v);
     }
+    for (int k = m & ~7; k < m; ++k) s.put(k, point(k, s.get(k)));
     return;
   }
 #pragma unroll 1
-  for (int k0 = 0; k0 < m; k0 += 8) {
-    uint64_t v[8];
-    s.load8(k0, v);
-#pragma unroll 1
-    for (int u = 0; u < 8; ++u) {
-      uint64_t t[4], b;
-      tab.row(k0 + u, t, b);
-      v[u] = pn::dbits(pn::corr_native(q, ew, v[u], t, st));
-    }
-    s.store8(k0, v);
+  for (int k = 0; k < m; ++k) {
+    uint64_t t[4], b;
+    tab.row(k, t, b);
+    s.put(k, pn::dbits(pn::corr_native(q, ew, s.get(k), t, st)));
   }
 }
 
@@ -830,22 +832,26 @@ __device__ __forceinline__ void correct_chunk(const pn::Par& q, const Tab& tab, 
 __device__ __forceinline__ double updated(double cbar, double v) { return cbar + v; }
 __device__ __forceinline__ float updated(float cbar, double v) { return narrow_rn(widen(cbar) + v); }
 
+// Words from one chunk to the next in shared memory: rows 2 modulo 4 (the lanes' 16-byte accesses then
+// fall on different banks), columns an odd number of rows.
+__host__ __device__ __forceinline__ int row_pitch(int m) { return m + ((6 - (m & 3)) & 3); }
+__host__ __device__ __forceinline__ int col_pitch(int m) { return m | 1; }
+
 // Whole lines in shared memory, both phases in one launch: the field is read once and written once.
-// Rows (COLS = 0): `lines` rows of n = P m values per block, one thread per (row, chunk); chunks padded
-// by 16 bytes so that the lanes' 16-byte accesses fall on different banks.
+// Rows: a few rows of n = P m values per block, one thread per (row, chunk).
 template <bool NF>
 __global__ void __launch_bounds__(64)
     k_line_rows(const double* __restrict__ in, double* __restrict__ out, const pn::Par q,
                             const LineTab lt, int P, int m, int vec) {
   extern __shared__ __align__(16) uint64_t sm[];
-  const int chunks = blockDim.x;  // lines * P
-  double2* sh = reinterpret_cast<double2*>(sm + static_cast<size_t>(chunks) * (m + 2));
+  const int chunks = blockDim.x, pitch = row_pitch(m);  // rows * P
+  double2* sh = reinterpret_cast<double2*>(sm + static_cast<size_t>(chunks) * pitch);
   const TabShared tab = stage_tables(reinterpret_cast<uint64_t*>(sh + chunks), lt, m);
   const int64_t base = static_cast<int64_t>(blockIdx.x) * chunks * m;  // consecutive rows are one range
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
   const int lanes = min(32, static_cast<int>(blockDim.x) - 32 * warp);
   for (int c = warp; c < chunks; c += nw) {
-    uint64_t* d = sm + c * (m + 2);
+    uint64_t* d = sm + c * pitch;
     const double* g = in + base + static_cast<int64_t>(c) * m;
     if (vec)
       for (int k = 2 * lane; k < m; k += 2 * lanes) cp_async16(d + k, g + k);
@@ -855,14 +861,14 @@ __global__ void __launch_bounds__(64)
   cp_async_wait();
   __syncthreads();
   const int p = threadIdx.x % P;
-  AccRow s{sm + threadIdx.x * (m + 2)};
+  AccRow s{sm + threadIdx.x * pitch};
   double ends[4], st[4];
   const int ew = pn::local_solve(q, s, s, m, ends);
   reduce_states<NF>(q, lt.mats, P, p, sh + (threadIdx.x - p), ends, st);
   correct_chunk(q, tab, s, m, ew, st);
   __syncthreads();
   for (int c = warp; c < chunks; c += nw) {
-    const double* d = reinterpret_cast<const double*>(sm + c * (m + 2));
+    const double* d = reinterpret_cast<const double*>(sm + c * pitch);
     double* g = out + base + static_cast<int64_t>(c) * m;
     if (vec)
       for (int k = 2 * lane; k < m; k += 2 * lanes) *reinterpret_cast<double2*>(g + k) = *reinterpret_cast<const double2*>(d + k);
@@ -886,9 +892,9 @@ __global__ void __launch_bounds__(256)
   constexpr int H = NC / 2;
   cg::cluster_group cluster = cg::this_cluster();
   const int CS = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
-  const int Pc = P / CS, threads = static_cast<int>(blockDim.x);  // Pc * NC
+  const int Pc = P / CS, threads = static_cast<int>(blockDim.x), pitch = col_pitch(m) * NC;  // Pc * NC threads
   // after the data: the scan's double2 per thread, then the end values (later the states), 4 per thread
-  double2* sh = reinterpret_cast<double2*>(sm + static_cast<size_t>(Pc) * (m + 1) * NC);
+  double2* sh = reinterpret_cast<double2*>(sm + static_cast<size_t>(Pc) * pitch);
   double* ex = reinterpret_cast<double*>(sh + threads);
   const TabShared tab = stage_tables(reinterpret_cast<uint64_t*>(ex + 4 * threads), lt, m);
   const int64_t x0 = static_cast<int64_t>(blockIdx.x / CS) * NC;
@@ -896,14 +902,14 @@ __global__ void __launch_bounds__(256)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (threads + 31) >> 5;
   const int lanes = min(32, threads - 32 * warp);
   for (int c = warp; c < Pc; c += nw) {
-    uint64_t* d = sm + c * (m + 1) * NC;
+    uint64_t* d = sm + c * pitch;
     const double* g = in + (row0 + static_cast<int64_t>(c) * m) * n + x0;
     for (int i = lane; i < m * H; i += lanes) cp_async16(d + 2 * i, g + static_cast<int64_t>(i / H) * n + 2 * (i % H));
   }
   cp_async_wait();
   __syncthreads();
   const int l = threadIdx.x % NC, c = threadIdx.x / NC;
-  AccCols<NC> s{sm + c * (m + 1) * NC + l};
+  AccCols<NC> s{sm + c * pitch + l};
   double ends[4], st[4];
   const int ew = pn::local_solve(q, s, s, m, ends);
 #pragma unroll
@@ -926,7 +932,7 @@ __global__ void __launch_bounds__(256)
   correct_chunk(q, tab, s, m, ew, st);
   __syncthreads();
   for (int cc = warp; cc < Pc; cc += nw) {
-    const double* d = reinterpret_cast<const double*>(sm + cc * (m + 1) * NC);
+    const double* d = reinterpret_cast<const double*>(sm + cc * pitch);
     T* g = next + (row0 + static_cast<int64_t>(cc) * m) * n + x0;
     for (int i0 = lane; i0 < m * H; i0 += 4 * lanes) {  // four pieces in flight
       using V = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
@@ -1013,6 +1019,11 @@ struct AccOut {  // reads W, writes the result of phase 2
       for (int u = 0; u < 8; ++u) next[(k + u) * es] = updated(cb[u], pn::from_bits(v[u]));
     }
   }
+  __device__ __forceinline__ uint64_t get(int k) const { return p[k * es]; }
+  __device__ __forceinline__ void put(int k, uint64_t v) const {
+    if constexpr (MODE == 0) out[k * es] = pn::from_bits(v);
+    else next[k * es] = updated(next[k * es], pn::from_bits(v));
+  }
 };
 
 // MODE 0 writes x (FP64) to out; MODE 1 adds it to Cbar in next.
@@ -1041,10 +1052,17 @@ bool valid_chunks(int64_t n, int P) {
 // are its chunks, and the scan over them costs what a few points do.  Rows + columns on GB300: 512^2
 // 34 us with 32 chunks (39 with 16), 1024^2 48 us with 32 (54 with 16, 56 with 64), 2048^2 114 us with
 // 64 (130 with 32), 4096^2 384 us with 64 (526 with 32).
+// Where that leaves chunks of more than 64 points (n = 64 times an odd number), any chunk length.
 int default_chunks(int64_t n) {
-  int P = 1;
-  while (valid_chunks(n, 2 * P) && n / (2 * P) >= (P < 32 ? 16 : 32)) P *= 2;
-  return P;
+  auto longest = [&](bool any) {
+    int P = 1;
+    while (2 * P <= pn::kMaxChunks && n % (2 * P) == 0 && (any || valid_chunks(n, 2 * P)) &&
+           n / (2 * P) >= (P < 32 ? 16 : 32))
+      P *= 2;
+    return P;
+  };
+  const int P = longest(false);
+  return n / P <= 64 ? P : longest(true);
 }
 
 // FP64 tiles (C^n, Cbar: halo 2; Z: halo 1), for either storage type.
@@ -1124,9 +1142,9 @@ int make_lines(int64_t n, int P, double a, bool noflux, int64_t scratch_lines, L
 // three or more share an SM and one's loads and stores run under the others' arithmetic.
 constexpr size_t kLineSmem = 75 * 1024, kLineSmemMax = 220 * 1024;
 
-// Rows per block (a row takes P (m + 2) words and the scan 2 P), 0 when a row does not fit; one or two
+// Rows per block (a row takes P row_pitch(m) words and the scan 2 P), 0 when a row does not fit; one or two
 // warps per block.
-size_t rows_smem(int P, int m, int k) { return static_cast<size_t>(k) * P * (8 * (m + 2) + 16) + kTabBytes * m; }
+size_t rows_smem(int P, int m, int k) { return static_cast<size_t>(k) * P * (8 * row_pitch(m) + 16) + kTabBytes * m; }
 int rows_per_block(int64_t rows, int P, int m) {
   int k = 1;
   while (k * P < 32 && k < 32) k *= 2;
@@ -1138,7 +1156,7 @@ int rows_per_block(int64_t rows, int P, int m) {
 // the chunks (eight at most), sixteen columns when that fits kLineSmem, else eight.
 struct ColShape { int nc, cs; };
 size_t cols_smem(int P, int m, ColShape s) {
-  return static_cast<size_t>(P / s.cs) * s.nc * (8 * (m + 1) + 16 + 32) + kTabBytes * m;
+  return static_cast<size_t>(P / s.cs) * s.nc * (8 * col_pitch(m) + 16 + 32) + kTabBytes * m;
 }
 ColShape cols_shape(int P, int m) {
   int cs = 8;
@@ -1165,7 +1183,7 @@ int launch_rows(const Lines& L, bool noflux, int64_t rows, const double* in, dou
   const int64_t n = static_cast<int64_t>(P) * m;
   const LineTab lt = line_tab(L);
   if (const int k = rows_per_block(rows, P, m)) {
-    const int vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
+    const int vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0 && m % 2 == 0;
     const unsigned grid = static_cast<unsigned>(rows / k);
     const size_t smem = rows_smem(P, m, k);
     if (noflux) k_line_rows<true><<<grid, k * P, smem, s>>>(in, out, L.par, lt, P, m, vec);

@@ -156,13 +156,14 @@ __host__ __device__ __forceinline__ void step(uint64_t& Y, uint64_t& D, uint64_t
   Y = Y + D - kBias;
 }
 
-// Phase 1 on one chunk, values at s (an accessor: load8 / store8 move 8 consecutive 64-bit words).
+// Phase 1 on one chunk, values at s (an accessor: load8 / store8 move 8 consecutive 64-bit words, get /
+// put one; the last m % 8 points are taken one by one).
 // Returns the scale mark: the exponent of W's unit, or kNative; ends = (y, D) / sqrt(c) after the
 // chunk and (W, E) / c before it.
 template <class Acc>
 __host__ __device__ __forceinline__ uint32_t chunk_max_hi(const Acc& s, int m) {
   uint32_t mx = 0;
-  for (int k0 = 0; k0 < m; k0 += 8) {
+  for (int k0 = 0; k0 + 8 <= m; k0 += 8) {
     uint64_t v[8];
     s.load8(k0, v);
 #pragma unroll
@@ -170,6 +171,10 @@ __host__ __device__ __forceinline__ uint32_t chunk_max_hi(const Acc& s, int m) {
       const uint32_t h = hi32(v[u]) & 0x7fffffffu;
       mx = h > mx ? h : mx;
     }
+  }
+  for (int k = m & ~7; k < m; ++k) {
+    const uint32_t h = hi32(s.get(k)) & 0x7fffffffu;
+    mx = h > mx ? h : mx;
   }
   return mx;
 }
@@ -181,7 +186,7 @@ __host__ __device__ __forceinline__ int local_fixed(const Par& q, const In& in, 
   const int E = 64 - q.nb + te;  // |b| < 2^(te - 1022)
   const int eu = te - 1022 - q.nb;  // exponent of y's unit
   uint64_t Y = kBias, D = kBias;
-  for (int k0 = 0; k0 < m; k0 += 8) {
+  for (int k0 = 0; k0 + 8 <= m; k0 += 8) {
     uint64_t v[8];
     in.load8(k0, v);
 #pragma unroll
@@ -191,15 +196,23 @@ __host__ __device__ __forceinline__ int local_fixed(const Par& q, const In& in, 
     }
     s.store8(k0, v);
   }
+  for (int k = m & ~7; k < m; ++k) {
+    step<WIDE>(Y, D, to_fixed(in.get(k), E), q.cn, q.ce, q.init_a, q.init_b, q.kc);
+    s.put(k, Y);
+  }
   ends[0] = static_cast<double>(static_cast<int64_t>(Y - kBias)) * (te ? q.eta * pow2(eu) : 0.0);
   ends[1] = static_cast<double>(static_cast<int64_t>(D - kBias)) * (te ? q.eta * pow2(eu) : 0.0);
   uint64_t W = kBias;
   D = kBias;
-  for (int k0 = m - 8; k0 >= 0; k0 -= 8) {
+  // from a zero state the first products are exact and make up for nothing: y is rounded there
+  s.put(m - 1, s.get(m - 1) + ((1ull << q.s2) >> 1));
+  for (int k = m - 1; k >= (m & ~7); --k) {
+    step<WIDE>(W, D, s.get(k) >> q.s2, q.cn, q.ce, q.init_a2, q.init_b, q.kc2);
+    s.put(k, W);
+  }
+  for (int k0 = (m & ~7) - 8; k0 >= 0; k0 -= 8) {
     uint64_t v[8];
     s.load8(k0, v);
-    // from a zero state the first products are exact and make up for nothing: y is rounded there
-    if (k0 == m - 8) v[7] += (1ull << q.s2) >> 1;
 #pragma unroll
     for (int u = 7; u >= 0; --u) {
       step<WIDE>(W, D, v[u] >> q.s2, q.cn, q.ce, q.init_a2, q.init_b, q.kc2);
@@ -217,7 +230,7 @@ template <class In, class Acc>
 __host__ __device__ __forceinline__ int local_native(const Par& q, const In& in, const Acc& s, int m,
                                                      double (&ends)[4]) {
   double Y = 0.0, D = 0.0;
-  for (int k0 = 0; k0 < m; k0 += 8) {
+  for (int k0 = 0; k0 + 8 <= m; k0 += 8) {
     uint64_t v[8];
     in.load8(k0, v);
 #pragma unroll 1
@@ -228,11 +241,21 @@ __host__ __device__ __forceinline__ int local_native(const Par& q, const In& in,
     }
     s.store8(k0, v);
   }
+  for (int k = m & ~7; k < m; ++k) {
+    D = D + (from_bits(in.get(k)) - fma(q.eta, Y, q.eps * D));
+    Y = Y + D;
+    s.put(k, dbits(Y));
+  }
   ends[0] = Y * q.eta;
   ends[1] = D * q.eta;
   double W = 0.0;
   D = 0.0;
-  for (int k0 = m - 8; k0 >= 0; k0 -= 8) {
+  for (int k = m - 1; k >= (m & ~7); --k) {
+    D = D + (from_bits(s.get(k)) - fma(q.eta, W, q.eps * D));
+    W = W + D;
+    s.put(k, dbits(W));
+  }
+  for (int k0 = (m & ~7) - 8; k0 >= 0; k0 -= 8) {
     uint64_t v[8];
     s.load8(k0, v);
 #pragma unroll 1
@@ -664,6 +687,8 @@ struct HostAcc {
   uint64_t* p;
   __host__ __device__ void load8(int k, uint64_t (&v)[8]) const { memcpy(v, p + k, 64); }
   __host__ __device__ void store8(int k, const uint64_t (&v)[8]) const { memcpy(p + k, v, 64); }
+  __host__ __device__ uint64_t get(int k) const { return p[k]; }
+  __host__ __device__ void put(int k, uint64_t v) const { p[k] = v; }
 };
 inline void solve_host(const Par& q, const std::vector<TabRow>& tab, const std::vector<uint64_t>& base,
                        const std::vector<double>& mats, int64_t n, int P, bool noflux, const double* b, double* x) {

@@ -38,7 +38,7 @@ def _residual(x, b, a, boundary):
 
 
 @pytest.mark.parametrize("boundary", [0, 1])
-@pytest.mark.parametrize("n, rows", [(64, 64), (128, 32), (320, 32), (512, 64), (1024, 32), (4096, 32), (8192, 32),
+@pytest.mark.parametrize("n, rows", [(64, 64), (128, 32), (320, 32), (512, 64), (1024, 32), (1472, 32), (2368, 32), (4096, 32), (8192, 32),
                                      (16384, 32), (32768, 32)])
 def test_rows_backward_error(env, n, rows, boundary):
     """|L x - b| <= 64 eps (1 + 16 a) max|x| per row (the bound the solver's host replay is held to), for
@@ -95,7 +95,7 @@ def test_rows_with_non_finite_values(env, n):
 
 @pytest.mark.parametrize("storage", [0, 1])
 @pytest.mark.parametrize("boundary", [0, 1])
-@pytest.mark.parametrize("n", [64, 512, 2048])
+@pytest.mark.parametrize("n", [64, 512, 1472, 2048, 2368])
 def test_column_kernels_equal_row_kernels(env, n, boundary, storage):
     """One full-grid step (columns by clusters of blocks) against its pieces on a band of all rows: the
     y lines by chunks through global memory, and through transposes as rows; fields bit for bit."""
