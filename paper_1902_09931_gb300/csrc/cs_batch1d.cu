@@ -238,6 +238,7 @@ __global__ void k_batch1d(const T* __restrict__ in, T* __restrict__ out,
   constexpr int kClamp = 1 << 30;
   constexpr int HL = LL > 0 ? LL : 1, HR = RR > 0 ? RR : 1;
 
+  overlap_wait();
   for (int64_t s0 = warp_id * kG; s0 < nseg; s0 += nwarps * kG) {  // warp-uniform loop
     T v[kG][E], hl[kG][HL], hr[kG][HR];
     int64_t m0[kG];
@@ -298,6 +299,7 @@ __global__ void k_batch1d_generic(const T* __restrict__ in, T* __restrict__ out,
                                   int64_t total, int64_t num_lines, int periodic, int L, int R,
                                   BTaps<T> taps) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  overlap_wait();
   for (int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; k < total; k += stride) {
     int64_t m = __ldg(seg + (k >> kSegShift));
     int64_t ls = __ldg(off + m), le = __ldg(off + m + 1);
@@ -330,9 +332,9 @@ int launch_t(const Batch1DConfig* c, const void* vin, void* vout, cudaStream_t s
   if constexpr (LL < 0) {
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((c->total_len + sh.threads - 1) / sh.threads,
                                                                 static_cast<int64_t>(num_sms()) * per_sm));
-    k_batch1d_generic<T><<<static_cast<unsigned>(grid), sh.threads, 0, st>>>(
+    CS_CUDA_TRY(launch_overlapped(k_batch1d_generic<T>, dim3(static_cast<unsigned>(grid)), dim3(sh.threads), 0, st, 
         in, out, c->d_offsets, c->d_seg_line, c->total_len, c->num_lines, c->bc == CS_BC_PERIODIC,
-        c->left, c->right, taps);
+        c->left, c->right, taps));
   } else {
     const int vec_ok = (reinterpret_cast<uintptr_t>(in) % 16 == 0) &&
                        (reinterpret_cast<uintptr_t>(out) % 16 == 0);
@@ -342,9 +344,9 @@ int launch_t(const Batch1DConfig* c, const void* vin, void* vout, cudaStream_t s
     int64_t grid = std::min<int64_t>((nseg + warps_per_cta * kG - 1) / (warps_per_cta * kG),
                                      static_cast<int64_t>(num_sms()) * per_sm);
     grid = std::max<int64_t>(grid, 1);
-    k_batch1d<T, LL, RR><<<static_cast<unsigned>(grid), sh.threads, 0, st>>>(
+    CS_CUDA_TRY(launch_overlapped(k_batch1d<T, LL, RR>, dim3(static_cast<unsigned>(grid)), dim3(sh.threads), 0, st, 
         in, out, c->d_offsets, c->d_seg_line, c->total_len, c->num_lines, c->bc == CS_BC_PERIODIC,
-        c->left, c->right, vec_ok, taps);
+        c->left, c->right, vec_ok, taps));
   }
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);

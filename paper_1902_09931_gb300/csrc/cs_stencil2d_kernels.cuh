@@ -386,6 +386,7 @@ __global__ void __launch_bounds__(kThreads)
   T* s = reinterpret_cast<T*>(smem_raw);
   const int64_t x0 = static_cast<int64_t>(blockIdx.x) * TX;
   const int64_t y0 = (static_cast<int64_t>(blockIdx.y) + ty0) * TY;
+  overlap_wait();
   load_tile_ct<T, ROWS, COLS>(s, in, nx, ny, periodic != 0, vec_ok != 0, x0, y0, sd.T, LA);
   if constexpr (sd.xform) xform_tile<T>(s, ROWS * COLS);
   spec_compute<T, TY, SPEC>(s, out, nx, ny, periodic, x0, y0, taps);
@@ -713,6 +714,7 @@ __global__ void __launch_bounds__(kThreads, ix_min_blocks(SPEC))
   }
   const int64_t x0 = bx * TX;
   const int64_t y0 = by * TY;
+  overlap_wait();
   load_tile_ct<double, ROWS, COLS>(s, in, nx, ny, periodic != 0, vec_ok != 0, x0, y0, sd.T, LA);
   // pass 1: the tile's largest exponent; inf / nan (and tiles outside the exponent window) take
   // native FP64
@@ -772,7 +774,7 @@ int launch_ix(const double* in, double* out, int64_t nx, int64_t ny, int periodi
   if (periodic || !whole || !cfg || !cfg->aux || ty0 != 0 || nty != nby || nbx < 3 || nby < 3) {
     auto kern = periodic && whole ? kfull : kedge;
     dim3 grid(static_cast<unsigned>(nbx), static_cast<unsigned>(nty));
-    kern<<<grid, kThreads, smem, st>>>(in, out, nx, ny, periodic, vec_ok, taps, itaps, 0, ty0, 0, 0);
+    CS_CUDA_TRY(launch_overlapped(kern, grid, dim3(kThreads), smem, st, in, out, nx, ny, periodic, vec_ok, taps, itaps, 0, ty0, 0, 0));
     CS_CUDA_TRY(cudaGetLastError());
     count_launches(1);
     return CS_OK;
@@ -843,6 +845,7 @@ __global__ void __launch_bounds__(kThreads) k_stencil2d_group(const __grid_const
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) unsigned s_red[kThreads / 32];
   T* s = reinterpret_cast<T*>(smem_raw);
+  overlap_wait();
   int j = 0;
   for (int b = static_cast<int>(blockIdx.x); b < tab.total_tiles; b += static_cast<int>(gridDim.x)) {
     while (j + 1 < tab.count && b >= tab.job[j + 1].tile_begin) ++j;
@@ -885,7 +888,7 @@ int launch_group(const GroupTable<T>& tab, cudaStream_t st) {
   }
   if (per_sm < 0) return set_error(CS_EUNSUPPORTED, "grouped stencil kernel does not fit on an SM");
   const int grid = static_cast<int>(std::min<int64_t>(tab.total_tiles, static_cast<int64_t>(num_sms()) * per_sm));
-  kern<<<static_cast<unsigned>(grid), kThreads, smem, st>>>(tab);
+  CS_CUDA_TRY(launch_overlapped(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreads), smem, st, tab));
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return CS_OK;
@@ -1160,6 +1163,7 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ int s_red[kThreads / 32];
   const int64_t x0 = static_cast<int64_t>(blockIdx.x) * TX;
   const int64_t y0 = (static_cast<int64_t>(blockIdx.y) + ty0) * TY;
+  overlap_wait();
   load_tile_ct<double, ROWS, COLS>(s, in, nx, ny, periodic != 0, vec_ok != 0, x0, y0, sd.T, LA);
   if constexpr (sd.xform) xform_tile<double>(s, ROWS * COLS);
   if (dd_split_tile<ROWS * COLS>(s, s_red))
@@ -1183,7 +1187,7 @@ int launch_dd(const double* in, double* out, int64_t nx, int64_t ny, int periodi
   window_tiles(TY, ny, &ty0, &nty);
   if (nty == 0) return CS_OK;
   dim3 grid(static_cast<unsigned>((nx + tile_x<double>() - 1) / tile_x<double>()), static_cast<unsigned>(nty));
-  kern<<<grid, kThreads, smem, st>>>(in, out, nx, ny, periodic, vec_ok, taps, dtaps, ty0);
+  CS_CUDA_TRY(launch_overlapped(kern, grid, dim3(kThreads), smem, st, in, out, nx, ny, periodic, vec_ok, taps, dtaps, ty0));
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return CS_OK;
@@ -1320,6 +1324,7 @@ __global__ void __launch_bounds__(kThreads)
     mbar_fence_init();
   }
   __syncthreads();
+  overlap_wait();
   auto issue = [&](int i, int st) {
     const int t = static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x);
     const int bx = t % tiles_x, by = t / tiles_x + ty0;
@@ -1401,9 +1406,9 @@ int launch_tma(const CUtensorMap& map, const T* in, T* out, int64_t nx, int64_t 
   if (tiles == 0) return CS_OK;
   if (tiles > 0x7fffffff) return set_error(CS_EINVAL, "grid too large for the TMA sweep");
   const int64_t grid = std::min<int64_t>(tiles, static_cast<int64_t>(num_sms()) * per_sm);
-  kern<<<static_cast<unsigned>(grid), kThreads, G::SMEM, st>>>(map, in, out, nx, ny, periodic,
+  CS_CUDA_TRY(launch_overlapped(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreads), G::SMEM, st, map, in, out, nx, ny, periodic,
                                                                static_cast<int>(tiles_x), static_cast<int>(tiles),
-                                                               ty0, taps, it, dt, status, stall_from);
+                                                               ty0, taps, it, dt, status, stall_from));
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return CS_OK;
@@ -1443,6 +1448,7 @@ __global__ void __launch_bounds__(kThreads)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* s = reinterpret_cast<T*>(smem_raw);
   T* ws = s + ROWS * COLS;
+  overlap_wait();
   for (int i = threadIdx.x; i < W * H; i += kThreads) ws[i] = wts[i];
 
   const int64_t x0 = static_cast<int64_t>(blockIdx.x) * TX;
@@ -1486,7 +1492,7 @@ int launch_spec(const T* in, T* out, int64_t nx, int64_t ny, int periodic, int v
   window_tiles(TY, ny, &ty0, &nty);
   if (nty == 0) return CS_OK;
   dim3 grid(static_cast<unsigned>((nx + tile_x<T>() - 1) / tile_x<T>()), static_cast<unsigned>(nty));
-  kern<<<grid, kThreads, smem, st>>>(in, out, nx, ny, periodic, vec_ok, taps, ty0);
+  CS_CUDA_TRY(launch_overlapped(kern, grid, dim3(kThreads), smem, st, in, out, nx, ny, periodic, vec_ok, taps, ty0));
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return CS_OK;
@@ -1510,8 +1516,8 @@ int launch_generic(const T* in, T* out, const Stencil2DConfig* cfg, const T* d_w
   window_tiles(TY, cfg->ny, &ty0, &nty);
   if (nty == 0) return CS_OK;
   dim3 grid(static_cast<unsigned>((cfg->nx + tile_x<T>() - 1) / tile_x<T>()), static_cast<unsigned>(nty));
-  kern<<<grid, kThreads, smem, st>>>(in, out, cfg->nx, cfg->ny, periodic, vec_ok, cfg->left,
-                                     cfg->right, cfg->top, cfg->bottom, d_w, xform, epi, ty0);
+  CS_CUDA_TRY(launch_overlapped(kern, grid, dim3(kThreads), smem, st, in, out, cfg->nx, cfg->ny, periodic, vec_ok, cfg->left,
+                                     cfg->right, cfg->top, cfg->bottom, d_w, xform, epi, ty0));
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   return CS_OK;

@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(kWThreads, sizeof(T) == 8 ? 4 : 1)
   __shared__ __align__(16) T s[kWTileRows * kWCols];
   const int64_t x0 = static_cast<int64_t>(blockIdx.x) * kWTX;
   const int64_t y0 = static_cast<int64_t>(blockIdx.y) * kWTY;
+  overlap_wait();
   s2d::load_tile<T>(s, c, nx, ny, true, vec_ok != 0, x0, y0, kWHalo, kWLA, kWCols, kWTileRows);
   const int tx = threadIdx.x % kWTX;
   const int r0 = (threadIdx.x / kWTX) * kWRows;
@@ -425,6 +426,7 @@ __global__ void __launch_bounds__(kWThreads)
   // so no row waits on a global load of its own; load_tile's wait covers all of them.  Edge tiles
   // (and unaligned u, v) read u and v per row from global memory.
   const bool staged = uv_ok && x0 + kW2TX <= nx && y0 + kWTY <= ny;
+  overlap_wait();
   if (staged) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     static_assert(kW2TX == 4 * 32, "one 16-byte chunk per lane and row");
@@ -517,15 +519,15 @@ int weno_launch(const WenoConfig* cfg, const void* c, const void* u, const void*
     }
     const int uv_ok = reinterpret_cast<uintptr_t>(u) % 16 == 0 && reinterpret_cast<uintptr_t>(v) % 16 == 0 &&
                       (cfg->nx * eb) % 16 == 0;
-    k_weno_adv_f32x2<<<grid, kWThreads, kW2Smem, st>>>(static_cast<const float*>(c), static_cast<const float*>(u),
+    CS_CUDA_TRY(launch_overlapped(k_weno_adv_f32x2, grid, dim3(kWThreads), kW2Smem, st, static_cast<const float*>(c), static_cast<const float*>(u),
                                                        static_cast<const float*>(v), static_cast<float*>(out),
                                                        cfg->nx, cfg->ny, vec_ok, uv_ok,
                                                        static_cast<float>(1.0 / cfg->hx),
-                                                       static_cast<float>(1.0 / cfg->hy));
+                                                       static_cast<float>(1.0 / cfg->hy)));
   } else {
-    k_weno_adv<double><<<grid, kWThreads, 0, st>>>(static_cast<const double*>(c), static_cast<const double*>(u),
+    CS_CUDA_TRY(launch_overlapped(k_weno_adv<double>, grid, dim3(kWThreads), 0, st, static_cast<const double*>(c), static_cast<const double*>(u),
                                                    static_cast<const double*>(v), static_cast<double*>(out), cfg->nx,
-                                                   cfg->ny, vec_ok, 1.0 / cfg->hx, 1.0 / cfg->hy, fx, fy);
+                                                   cfg->ny, vec_ok, 1.0 / cfg->hx, 1.0 / cfg->hy, fx, fy));
   }
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
