@@ -17,10 +17,12 @@
 // untouched.  Stencils wider than the vector width take a per-element kernel.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 
 #include "cs_internal.h"
+#include "cs_penta.cuh"
 
 namespace cs {
 namespace {
@@ -32,6 +34,59 @@ template <> struct Vec1<float> { static constexpr int n = 4; using V = float4; }
 template <> struct Vec1<double> { static constexpr int n = 2; using V = double2; };
 
 template <typename T> struct BTaps { T w[2 * CS_MAX_EXTENT + 1]; };
+
+// Weights as c (n_k + rho_k): integers n_k, sum |n_k| <= 64, |rho_k| small; c = cm 2^(ce - 64).
+struct IxLine {
+  int32_t n[5];
+  float rho[5];  // in units of the fixed-point sum per 2^32 of the value
+  int32_t ok, exact, ce;
+  int32_t bits;  // fixed-point bits of a value: the sum takes log2 of sum |n_k| more, 62 in all
+  uint64_t cm;
+};
+
+// The fixed-point form of a radius-2 stencil's weights, ok = 0 when they have none (no common scale to
+// 2^-44 of the largest weight, as the 2D sweeps' digit path asks, or one outside 2^[-100, 100]).
+IxLine line_ratios(const Batch1DConfig* c) {
+  IxLine ix;
+  memset(&ix, 0, sizeof ix);
+  const int W = c->left + c->right + 1;
+  if (c->dtype != CS_F64 || c->left > 2 || c->right > 2) return ix;
+  double wmin = 0.0, wmax = 0.0;
+  for (int i = 0; i < W; ++i) {
+    const double a = std::fabs(c->weights[i]);
+    if (!(a <= 0x1p100) || (a > 0.0 && a < 0x1p-100)) return ix;
+    if (a > 0.0 && (wmin == 0.0 || a < wmin)) wmin = a;
+    if (a > wmax) wmax = a;
+  }
+  if (wmax == 0.0) return ix;
+  for (int m = 1; m <= 64; ++m) {
+    const double q = wmin / m;
+    long long total = 0;
+    bool fits = true;
+    for (int i = 0; i < W && fits; ++i) {
+      const long long k = std::llround(c->weights[i] / q);
+      fits = std::fabs(c->weights[i] - static_cast<double>(k) * q) <= 0x1p-44 * wmax;
+      total += k < 0 ? -k : k;
+      fits = fits && total <= 64;
+      ix.n[i] = static_cast<int32_t>(k);
+    }
+    if (!fits) continue;
+    ix.ok = ix.exact = 1;
+    ix.bits = 62;
+    for (long long t = 1; t < total; t *= 2) --ix.bits;
+    int e;
+    std::frexp(q, &e);  // q in [2^(e-1), 2^e)
+    ix.cm = static_cast<uint64_t>(std::ldexp(q, 53 - e)) << 11;
+    ix.ce = e;
+    for (int i = 0; i < W; ++i) {
+      const double r = std::fma(-static_cast<double>(ix.n[i]), q, c->weights[i]) / q;  // exact difference
+      ix.rho[i] = static_cast<float>(r * 0x1p32);
+      if (r != 0.0) ix.exact = 0;
+    }
+    return ix;
+  }
+  return ix;
+}
 
 struct LaunchShape { int threads, ctas_per_sm; };
 constexpr LaunchShape kShapes[] = {{256, 4}, {256, 8}, {512, 2}, {128, 8}, {512, 1}, {256, 2}};
@@ -88,6 +143,62 @@ __device__ __forceinline__ void elements_general(const T* __restrict__ in, T* __
 constexpr int kLaneVecs = 2;
 template <typename T> constexpr int lane_elems() { return kLaneVecs * Vec1<T>::n; }
 
+// Writes a lane's E results of the segment at s.  r0 .. r3: the boundaries off[m0] .. off[m0 + 3]
+// relative to s (clamped; total past the last line), m0 the line of s.  An element is written
+// only when its stencil stays inside its line.
+template <typename T, int L, int R, int E>
+__device__ __forceinline__ void write_segment(T* __restrict__ out, const int64_t* __restrict__ off, int64_t total,
+                                              bool vec_ok, int64_t s, int64_t m0, int r0, int r1, int r2, int r3,
+                                              const T (&res)[E]) {
+  constexpr int V = Vec1<T>::n;
+  using VT = typename Vec1<T>::V;
+  const int lane = threadIdx.x & 31;
+  const int64_t k0 = s + lane * E;
+  const int o = lane * E, oe = o + E - 1;
+  const int c0 = (o >= r1) + (o >= r2), c1 = (oe >= r1) + (oe >= r2);
+  const int ls = c0 == 0 ? r0 : (c0 == 1 ? r1 : r2);
+  const int le = c0 == 0 ? r1 : (c0 == 1 ? r2 : r3);
+  if (c0 == c1 && oe < r3 && k0 + E <= total && o - L >= ls && oe + R < le) {  // the common case
+    if (vec_ok) {
+#pragma unroll
+      for (int q = 0; q < E / V; ++q) {
+        VT y;
+        if constexpr (V == 4) { y.x = res[4 * q]; y.y = res[4 * q + 1]; y.z = res[4 * q + 2]; y.w = res[4 * q + 3]; }
+        else { y.x = res[2 * q]; y.y = res[2 * q + 1]; }
+        *reinterpret_cast<VT*>(out + k0 + q * V) = y;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; ++e) out[k0 + e] = res[e];
+    }
+    return;
+  }
+  if (oe < r3) {  // near a line end: each element's line is one of the segment's three
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int oo = o + e;
+      const int ce = (oo >= r1) + (oo >= r2);
+      const int ls_e = ce == 0 ? r0 : (ce == 1 ? r1 : r2);
+      const int le_e = ce == 0 ? r1 : (ce == 1 ? r2 : r3);
+      if (k0 + e < total && oo - ls_e >= L && le_e - 1 - oo >= R) out[k0 + e] = res[e];
+    }
+    return;
+  }
+  // more lines in this segment than its four boundaries describe (lines shorter than a
+  // segment): walk the offsets from the lane's first line
+  int64_t m = m0 + c0, lsa = s + ls, lea = s + le;
+  for (int e = 0; e < E; ++e) {
+    const int64_t k = k0 + e;
+    if (k >= total) break;
+    while (k >= lea) {  // skips empty lines
+      ++m;
+      lsa = lea;
+      lea = __ldg(off + m + 1);
+    }
+    if (k - lsa >= L && lea - 1 - k >= R) out[k] = res[e];
+  }
+}
+
 // One warp segment of 32 * E packed elements starting at s: own values v (already loaded),
 // neighbours by shuffle (lanes 0 and 31 take the nearest L / R values of the adjacent segments
 // from hl / hr, loaded with the segment), the lane's line from the segment's boundaries, and the
@@ -137,49 +248,7 @@ __device__ __forceinline__ void segment(const T* __restrict__ in, T* __restrict_
     for (int p = 0; p < W; ++p) acc = fma(taps.w[p], win[e + p], acc);
     res[e] = acc;
   }
-  const int o = lane * E, oe = o + E - 1;
-  const int c0 = (o >= r1) + (o >= r2), c1 = (oe >= r1) + (oe >= r2);
-  const int ls = c0 == 0 ? r0 : (c0 == 1 ? r1 : r2);
-  const int le = c0 == 0 ? r1 : (c0 == 1 ? r2 : r3);
-  if (c0 == c1 && oe < r3 && k0 + E <= total && o - L >= ls && oe + R < le) {  // the common case
-    if (vec_ok) {
-#pragma unroll
-      for (int q = 0; q < kLaneVecs; ++q) {
-        VT y;
-        if constexpr (V == 4) { y.x = res[4 * q]; y.y = res[4 * q + 1]; y.z = res[4 * q + 2]; y.w = res[4 * q + 3]; }
-        else { y.x = res[2 * q]; y.y = res[2 * q + 1]; }
-        *reinterpret_cast<VT*>(out + k0 + q * V) = y;
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < E; ++e) out[k0 + e] = res[e];
-    }
-    return;
-  }
-  if (oe < r3) {  // near a line end: each element's line is one of the segment's three
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int oo = o + e;
-      const int ce = (oo >= r1) + (oo >= r2);
-      const int ls_e = ce == 0 ? r0 : (ce == 1 ? r1 : r2);
-      const int le_e = ce == 0 ? r1 : (ce == 1 ? r2 : r3);
-      if (k0 + e < total && oo - ls_e >= L && le_e - 1 - oo >= R) out[k0 + e] = res[e];
-    }
-    return;
-  }
-  // more lines in this segment than its four boundaries describe (lines shorter than a
-  // segment): walk the offsets from the lane's first line
-  int64_t m = m0 + c0, lsa = s + ls, lea = s + le;
-  for (int e = 0; e < E; ++e) {
-    const int64_t k = k0 + e;
-    if (k >= total) break;
-    while (k >= lea) {  // skips empty lines
-      ++m;
-      lsa = lea;
-      lea = __ldg(off + m + 1);
-    }
-    if (k - lsa >= L && lea - 1 - k >= R) out[k] = res[e];
-  }
+  write_segment<T, LL, RR, E>(out, off, total, vec_ok, s, m0, r0, r1, r2, r3, res);
 }
 
 // The first L and last R elements of every periodic line, whose stencils wrap around the line:
@@ -292,6 +361,151 @@ __global__ void k_batch1d(const T* __restrict__ in, T* __restrict__ out,
                  static_cast<int64_t>(gridDim.x) * blockDim.x);
 }
 
+// FP64 lines whose weights are c n_k with integers n_k, sum |n_k| <= 64, in 64-bit fixed point.  At two
+// FP64 instructions per clock and SM the five multiply-adds of a radius-2 stencil bound the FP64 walk at
+// 634 us for 63.5 M elements (FP32 storage 84 us; the floor of 16 bytes an element is 150 us).  Now 263 us,
+// bound by latency and the integer pipes (99 instructions an element).  Here a warp segment's
+// values become integers of 56 to 62 bits of its largest (62 with the bits that the sum takes), the
+// weighted sums are exact, and the one FP64 instruction left converts the scaled sum; what the weights miss of
+// c n_k joins the sum as an integer formed in FP32 (IxLine::rho), so the weights are the caller's to
+// 2^-60.  The result is the exact sum of the rounded inputs rounded twice, where the FMA chain rounds each
+// partial sum: error against 64-bit reference lines no larger (tests/test_gpu_batch1d_fixed.py).
+// 8 elements per lane, so that the two neighbours a lane of the segment's ends converts are shared by 8.
+// Segments that hold infinities, NaN or only values outside 2^[-860, 870] take the FP64 chain.
+constexpr int kIxElems = 8;
+constexpr int kIxMinE = 160;  // with |c| >= 2^-100 no result is subnormal
+
+template <int L, int R>
+__global__ void __launch_bounds__(256, 3)
+    k_batch1d_ix(const double* __restrict__ in, double* __restrict__ out, const int64_t* __restrict__ off,
+                 const int32_t* __restrict__ seg, int64_t total, int64_t num_lines, int periodic, int vec_ok,
+                 BTaps<double> taps, IxLine ix) {
+  constexpr int E = kIxElems, W = L + R + 1, H = L > R ? L : R;
+  const int lane = threadIdx.x & 31;
+  const int64_t warp_id = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+  constexpr int64_t kSeg = 32 * E;
+  static_assert(kSeg % (int64_t(1) << kSegShift) == 0, "segments start on line-table entries");
+  const int64_t nseg = (total + kSeg - 1) / kSeg;
+  constexpr int kClamp = 1 << 30;
+
+  overlap_wait();
+  // a segment's loads: its values, the H values before it (lane 0) or after it (lane 31), its first line
+  // and the boundaries from there (lanes 0..3); the next segment's are issued before this one's arithmetic
+  double nv[E], nh[H > 0 ? H : 1];
+  int64_t nm0 = 0;
+  auto fetch = [&](int64_t sg) {
+    const int64_t s = sg * kSeg, k0 = s + lane * E;
+    if (sg >= nseg) return;
+    nm0 = __ldg(seg + (s >> kSegShift));
+    if (vec_ok && k0 + E <= total) {
+#pragma unroll
+      for (int q = 0; q < E; q += 2) {
+        const double2 x = *reinterpret_cast<const double2*>(in + k0 + q);
+        nv[q] = x.x;
+        nv[q + 1] = x.y;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < E; ++e) nv[e] = k0 + e < total ? in[k0 + e] : 0.0;
+    }
+#pragma unroll
+    for (int e = 0; e < H; ++e) {
+      const int64_t k = lane == 0 ? k0 - H + e : k0 + E + e;
+      nh[e] = (lane == 0 || lane == 31) && k >= 0 && k < total ? __ldg(in + k) : 0.0;
+    }
+  };
+  fetch(warp_id);
+  for (int64_t sg = warp_id; sg < nseg; sg += nwarps) {  // warp-uniform loop
+    const int64_t s = sg * kSeg, k0 = s + lane * E;
+    double v[E], h[H > 0 ? H : 1];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = nv[e];
+#pragma unroll
+    for (int e = 0; e < H; ++e) h[e] = nh[e];
+    const int64_t m0 = nm0;
+    const int64_t b = (lane < 4 && m0 + lane <= num_lines) ? __ldg(off + m0 + lane) : total;
+    fetch(sg + nwarps);
+    uint32_t mx = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) mx = max(mx, pn::hi32(pn::dbits(v[e])) & 0x7fffffffu);
+#pragma unroll
+    for (int e = 0; e < H; ++e) mx = max(mx, pn::hi32(pn::dbits(h[e])) & 0x7fffffffu);
+    const int te = static_cast<int>(__reduce_max_sync(0xffffffffu, mx) >> 20);
+    double res[E];
+    if (te >= kIxMinE && te <= pn::kMaxE) {
+      const int sh = 64 - ix.bits + te;
+      int64_t win[E + 2 * H];
+#pragma unroll
+      for (int e = 0; e < E; ++e) win[H + e] = static_cast<int64_t>(pn::to_fixed(pn::dbits(v[e]), sh));
+#pragma unroll
+      for (int e = 0; e < H; ++e) {
+        const long long own = static_cast<long long>(pn::to_fixed(pn::dbits(h[e]), sh));
+        const long long left = __shfl_up_sync(0xffffffffu, static_cast<long long>(win[H + E - H + e]), 1);
+        const long long right = __shfl_down_sync(0xffffffffu, static_cast<long long>(win[H + e]), 1);
+        win[e] = lane == 0 ? own : left;
+        win[H + E + e] = lane == 31 ? own : right;
+      }
+      int64_t sum[E];
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        int64_t acc = 0;
+#pragma unroll
+        for (int p = 0; p < W; ++p) acc += ix.n[p] * win[H - L + e + p];
+        sum[e] = acc;
+      }
+      if (ix.exact == 0) {
+        float f[E + 2 * H];
+#pragma unroll
+        for (int e = 0; e < E + 2 * H; ++e) f[e] = __int2float_rn(static_cast<int>(win[e] >> 32));
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          float c = 0.0f;
+#pragma unroll
+          for (int p = 0; p < W; ++p) c = fmaf(ix.rho[p], f[H - L + e + p], c);
+          sum[e] += __float2int_rn(c);
+        }
+      }
+      // sum c: the high 64 bits of the biased product, the bias's own share (cm is a multiple of 4) taken off
+      const uint32_t ch = pn::hi32(ix.cm), cl = pn::lo32(ix.cm);
+      const uint64_t ex = static_cast<uint64_t>(static_cast<uint32_t>(ix.ce + te - 1022 - ix.bits)) << 52;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const uint64_t u = static_cast<uint64_t>(sum[e]) + pn::kBias;
+        const uint64_t lo = pn::wmul(pn::lo32(u), ch) + 0x80000000ull;
+        const uint64_t T = pn::wmul(pn::hi32(u), ch) + pn::hi32(lo) + pn::mad_hi(pn::hi32(u), cl, 0u) - (ix.cm >> 2);
+        const double x = __ll2double_rn(static_cast<long long>(T));
+        res[e] = T ? pn::from_bits(pn::dbits(x) + ex) : 0.0;
+      }
+    } else {
+      double win[E + 2 * H];
+#pragma unroll
+      for (int e = 0; e < E; ++e) win[H + e] = v[e];
+#pragma unroll
+      for (int e = 0; e < H; ++e) {
+        const double left = __shfl_up_sync(0xffffffffu, v[E - H + e], 1), right = __shfl_down_sync(0xffffffffu, v[e], 1);
+        win[e] = lane == 0 ? h[e] : left;
+        win[H + E + e] = lane == 31 ? h[e] : right;
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        double acc = 0.0;
+#pragma unroll
+        for (int p = 0; p < W; ++p) acc = fma(taps.w[p], win[H - L + e + p], acc);
+        res[e] = acc;
+      }
+    }
+    const int64_t d = b - s;
+    const int r = static_cast<int>(d < -kClamp ? -kClamp : (d > kClamp ? kClamp : d));
+    const int r0 = __shfl_sync(0xffffffffu, r, 0), r1 = __shfl_sync(0xffffffffu, r, 1);
+    const int r2 = __shfl_sync(0xffffffffu, r, 2), r3 = __shfl_sync(0xffffffffu, r, 3);
+    if (k0 < total) write_segment<double, L, R, E>(out, off, total, vec_ok != 0, s, m0, r0, r1, r2, r3, res);
+  }
+  if (periodic && L + R > 0)
+    line_ends<double>(in, out, off, num_lines, L, R, taps, static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x,
+                      static_cast<int64_t>(gridDim.x) * blockDim.x);
+}
+
 // Any extents up to CS_MAX_EXTENT: every element on its own, lines found through the table.
 template <typename T>
 __global__ void k_batch1d_generic(const T* __restrict__ in, T* __restrict__ out,
@@ -338,6 +552,20 @@ int launch_t(const Batch1DConfig* c, const void* vin, void* vout, cudaStream_t s
   } else {
     const int vec_ok = (reinterpret_cast<uintptr_t>(in) % 16 == 0) &&
                        (reinterpret_cast<uintptr_t>(out) % 16 == 0);
+    if constexpr (sizeof(T) == 8) {
+      const IxLine ix = line_ratios(c);
+      if (ix.ok) {
+        int fit = 0;
+        CS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_batch1d_ix<LL, RR>, 256, 0));
+        const int64_t nseg = (c->total_len + 32 * kIxElems - 1) / (32 * kIxElems);
+        const int64_t grid = std::min<int64_t>((nseg + 7) / 8, static_cast<int64_t>(num_sms()) * std::max(fit, 1));
+        CS_CUDA_TRY(launch_overlapped(k_batch1d_ix<LL, RR>, dim3(static_cast<unsigned>(std::max<int64_t>(grid, 1))), dim3(256),
+                                      0, st, in, out, c->d_offsets, c->d_seg_line, c->total_len, c->num_lines,
+                                      c->bc == CS_BC_PERIODIC, vec_ok, taps, ix));
+        count_launches(1);
+        return CS_OK;
+      }
+    }
     const int64_t seg_elems = 32 * lane_elems<T>();
     const int64_t nseg = (c->total_len + seg_elems - 1) / seg_elems;
     const int64_t warps_per_cta = sh.threads / 32;
