@@ -100,7 +100,7 @@ _SYMBOLS = {
     "cs_plan_create_1d_batch": (ctypes.c_int, [ctypes.POINTER(ctypes.c_void_p), ctypes.POINTER(_CStencilDesc), ctypes.c_int64, ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p]),
     "cs_compute": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
     "cs_compute_host": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
-    "cs_compute_group": (ctypes.c_int, [ctypes.POINTER(ctypes.c_void_p), ctypes.c_int32, ctypes.c_void_p]),
+    "cs_compute_group": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p]),  # an array of handles
     "cs_swap": (ctypes.c_int, [ctypes.c_void_p]),
     "cs_set_buffers": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
     "cs_plan_use_graph": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
@@ -166,10 +166,27 @@ def _ptr(x) -> int:
     raise TypeError(f"cannot take the address of {type(x)}")
 
 
+_raw_stream = None  # () -> handle of torch's current stream
+
+
+def _current_stream() -> int:
+    """The handle of torch's current stream, from the raw query where torch has it (a stream object per
+    call cost more than the rest of a small sweep's call)."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        query, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if query is not None and device is not None and torch.cuda.is_available():
+            torch.cuda.current_stream()  # initialises the context
+            _raw_stream = lambda: query(device())
+        else:
+            _raw_stream = lambda: int(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream()
+
+
 def _stream(s) -> int:
     if s is None:
-        import torch
-        return int(torch.cuda.current_stream().cuda_stream)
+        return _current_stream()
     if isinstance(s, int):
         return s
     if hasattr(s, "cuda_stream"):
@@ -242,13 +259,18 @@ def cs_plan_create_1d_batch(desc: StencilDesc, num_lines: int, d_offsets, total_
 
 
 def cs_compute(plan, stream=None) -> None:
-    _check(load().cs_compute(plan, _stream(stream)))
+    rc = (_lib or load()).cs_compute(plan, _current_stream() if stream is None else _stream(stream))
+    if rc:
+        _check(rc)
 
 
 def cs_compute_group(plans, stream=None) -> None:
-    """One grouped launch (per 16 plans) over several 2D stencil plans of the same shape."""
-    arr = (ctypes.c_void_p * len(plans))(*[p.value if hasattr(p, "value") else p for p in plans])
-    _check(load().cs_compute_group(arr, len(plans), _stream(stream)))
+    """One grouped launch (per 64 plans) over several 2D stencil plans of the same shape."""
+    try:
+        arr = b"".join(plans)  # the handles' own bytes: c_void_p objects are buffers
+    except TypeError:  # plain addresses among them
+        arr = (ctypes.c_void_p * len(plans))(*[p.value if hasattr(p, "value") else p for p in plans])
+    _check((_lib or load()).cs_compute_group(arr, len(plans), _stream(stream)))
 
 
 def cs_compute_host(plan, h_in, h_out, stream=None) -> None:

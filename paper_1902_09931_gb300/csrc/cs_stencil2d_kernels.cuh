@@ -16,6 +16,7 @@
 // kernel takes any extents up to CS_MAX_EXTENT at run time.
 #pragma once
 
+#include <type_traits>
 #include <cuda.h>
 #include <stdint.h>
 #include <string.h>
@@ -822,13 +823,14 @@ int dispatch_ix(int variant, const double* in, double* out, int64_t nx, int64_t 
 // CUDA graph.
 constexpr int kMaxGroup = 64;
 
+struct NoIxTaps {};
 template <typename T> struct GroupJob {
   const T* in;
   T* out;
   int64_t nx, ny;
   int tiles_x, tile_begin, periodic, vec_ok;
   Taps<T> taps;
-  IxTaps itaps;
+  typename std::conditional<sizeof(T) == 8, IxTaps, NoIxTaps>::type itaps;  // digit path: FP64 storage only
 };
 template <typename T> struct GroupTable {
   int count, total_tiles;
@@ -913,8 +915,8 @@ int dispatch_group(int variant, const GroupTable<T>& tab, cudaStream_t st) {
 template <typename T>
 int launch_group_t(const Stencil2DConfig* const* cfgs, const void* const* ins, void* const* outs,
                    int count, cudaStream_t st) {
-  GroupTable<T> tab;
-  memset(&tab, 0, sizeof tab);
+  GroupTable<T> tab;  // count jobs of it are filled and read
+  tab.count = 0;
   // FP32 storage gives the same bits with either tile height: 32 rows, so that a batch of small grids
   // spreads over twice the CTAs
   const int variant = cfgs[0]->variant, TY = sizeof(T) == 4 ? 32 : cfgs[0]->tile_rows;
@@ -940,12 +942,15 @@ int launch_group_t(const Stencil2DConfig* const* cfgs, const void* const* ins, v
     g.vec_ok = (c->nx % Vec<T>::n == 0) && (reinterpret_cast<uintptr_t>(ins[j]) % 16 == 0);
     for (int i = 0; i < 32; ++i) g.taps.w[i] = i < nt ? static_cast<T>(c->weights[i]) : T(0);
     digits = digits && c->ix_ok && c->fp64_mode == CS_FP64_AUTO;
-    for (int i = 0; i < 32; ++i) g.itaps.n[i] = static_cast<int8_t>(i < nt && c->ix_ok ? c->ix_n[i] : 0);
-    g.itaps.c = ixd::ixi_round51(c->ix_c);
-    g.itaps.c15 = -1.5 * g.itaps.c;
-    if (c->ix_ok) {
-      g.itaps.inv_hi = static_cast<float>(1.0 / c->ix_c);
-      g.itaps.inv_lo = static_cast<float>(1.0 / c->ix_c - static_cast<double>(g.itaps.inv_hi));
+    if constexpr (sizeof(T) == 8) {
+      g.itaps = IxTaps{};
+      if (c->ix_ok) {
+        for (int i = 0; i < nt; ++i) g.itaps.n[i] = static_cast<int8_t>(c->ix_n[i]);
+        g.itaps.c = ixd::ixi_round51(c->ix_c);
+        g.itaps.c15 = -1.5 * g.itaps.c;
+        g.itaps.inv_hi = static_cast<float>(1.0 / c->ix_c);
+        g.itaps.inv_lo = static_cast<float>(1.0 / c->ix_c - static_cast<double>(g.itaps.inv_hi));
+      }
     }
     ++tab.count;
   }
