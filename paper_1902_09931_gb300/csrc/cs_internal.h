@@ -26,8 +26,8 @@ int num_sms();                   // SM count of the current device (cached per d
 // Launches a kernel that begins with overlap_wait(): its blocks may become resident while the stream's
 // previous kernel drains, and wait there until that kernel has completed and its writes are visible, so
 // stream order holds as ever; only the launch latency and the previous kernel's last wave are
-// overlapped.  4096^2 back to back: FP32 9-point Laplacian 25.5 -> 23.9 us, FP64 cubic user function 59.7 ->
-// 57.6 us.  Not used by the Cahn-Hilliard step, whose kernels replay from a graph: 1024^2 63 -> 72 us.
+// overlapped.  4096^2 back to back: FP32 9-point Laplacian 25.5 -> 23.9 us, FP64 cubic user function 59.5 ->
+// 57.3 us.  Not used by the Cahn-Hilliard step, whose kernels replay from a graph: 1024^2 63 -> 72 us.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_overlapped(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                      Args... args) {

@@ -123,7 +123,10 @@ __device__ __forceinline__ void load_tile_interior(T* s, const T* __restrict__ i
   __syncthreads();
 }
 
-template <typename T>
+// COMPACT: the edge tiles' copy as one rolled loop, for kernels whose registers are capped and whose
+// edge tiles are few (the FULL digit kernel: the unrolled loops below spilled its weights, 8192^2
+// biharmonic 206.2 us with them, 201.2 with the rolled one).
+template <typename T, bool COMPACT = false>
 __device__ __forceinline__ void load_tile(T* s, const T* __restrict__ in, int64_t nx, int64_t ny,
                                           bool periodic, bool vec_ok, int64_t x0, int64_t y0,
                                           int top, int LA, int cols, int rows) {
@@ -154,6 +157,32 @@ __device__ __forceinline__ void load_tile(T* s, const T* __restrict__ in, int64_
   // element by element, without the wraps where the tile lies inside the grid.
   const bool one_wrap = nx >= cols && ny >= rows;  // tile halo reaches at most one period out
   auto wrapped = [&](int64_t k, int64_t n) { return one_wrap ? (k < 0 ? k + n : (k >= n ? k - n : k)) : wrap_idx(k, n); };
+  if constexpr (COMPACT) {
+#pragma unroll 1
+    for (int idx = threadIdx.x; idx < total; idx += kThreads) {
+      const int r = idx / nch, ch = idx - r * nch;
+      int64_t gy = gy0 + r, gx = gx0 + static_cast<int64_t>(ch) * V;
+      T* dst = s + r * cols + ch * V;
+      if (vec_ok) {
+        const bool inside = gy >= 0 && gy < ny && gx >= 0 && gx < nx;
+        if (inside || periodic)
+          cp_async16(dst, in + wrapped(gy, ny) * nx + wrapped(gx, nx));
+        else
+          *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+        for (int e = 0; e < V; ++e, ++gx) {
+          const bool inside = gy >= 0 && gy < ny && gx >= 0 && gx < nx;
+          if (inside || periodic)
+            cp_async_elem(dst + e, in + wrapped(gy, ny) * nx + wrapped(gx, nx));
+          else
+            dst[e] = T(0);
+        }
+      }
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    return;
+  }
   if (vec_ok) {
 #pragma unroll 4
     for (int idx = threadIdx.x; idx < total; idx += kThreads) {
@@ -200,7 +229,7 @@ __device__ __forceinline__ void load_tile(T* s, const T* __restrict__ in, int64_
 }
 
 // load_tile for a compile-time tile shape: interior tiles take the unrolled copy.
-template <typename T, int ROWS, int COLS>
+template <typename T, int ROWS, int COLS, bool COMPACT = false>
 __device__ __forceinline__ void load_tile_ct(T* s, const T* __restrict__ in, int64_t nx, int64_t ny,
                                              bool periodic, bool vec_ok, int64_t x0, int64_t y0,
                                              int top, int LA) {
@@ -209,7 +238,7 @@ __device__ __forceinline__ void load_tile_ct(T* s, const T* __restrict__ in, int
     load_tile_interior<T, ROWS, COLS>(s, in, nx, gy0, gx0);
     return;
   }
-  load_tile<T>(s, in, nx, ny, periodic, vec_ok, x0, y0, top, LA, COLS, ROWS);
+  load_tile<T, COMPACT>(s, in, nx, ny, periodic, vec_ok, x0, y0, top, LA, COLS, ROWS);
 }
 
 template <typename T>
@@ -716,7 +745,7 @@ __global__ void __launch_bounds__(kThreads, ix_min_blocks(SPEC))
   const int64_t x0 = bx * TX;
   const int64_t y0 = by * TY;
   overlap_wait();
-  load_tile_ct<double, ROWS, COLS>(s, in, nx, ny, periodic != 0, vec_ok != 0, x0, y0, sd.T, LA);
+  load_tile_ct<double, ROWS, COLS, FULL>(s, in, nx, ny, periodic != 0, vec_ok != 0, x0, y0, sd.T, LA);
   // pass 1: the tile's largest exponent; inf / nan (and tiles outside the exponent window) take
   // native FP64
   const uint32_t mhi = ixd::ix_tile_max_hi<kThreads, ROWS * COLS>(s, s_red);
@@ -1551,7 +1580,7 @@ int make_tensor_map(const Stencil2DConfig* cfg, const void* in, int elem_bytes, 
 //   FP64 storage on the digit or double-float path: tiles of 32 rows up to 2^22.5 points, where more
 //   CTAs hide each other's load and reduction phases (9-point Laplacian, 256^2 3.8 against 5.4 with 64
 //   rows and 5.7 with TMA; 2048^2 18.2 / 19.8 / 20.9; 3072^2 34.9 / 34.6 / 38.5), 64 rows beyond
-//   (4096^2 57.6 / 54.6 / 61.4; 8192^2 biharmonic 230 / 203 / 240), and 32 rows for rows that are not
+//   (4096^2 57.6 / 54.6 / 61.4; 8192^2 biharmonic 230 / 201 / 240), and 32 rows for rows that are not
 //   16-byte aligned (4097^2 69.0 / 77.2);
 //   FP32 storage: 32 rows (512^2 2.7 / 3.5 / 4.0; 4096^2 23.7 / 24.1 / 24.3; 8192^2 84.5 / 84.0 /
 //   94.8; 4097^2 32.1 / 38.3), except TMA for non-periodic stencils that reach sideways on 2^20 to
