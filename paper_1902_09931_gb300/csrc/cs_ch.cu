@@ -819,6 +819,11 @@ __device__ __forceinline__ void correct_chunk(const pn::Par& q, const Tab& tab, 
     for (int k = m & ~7; k < m; ++k) s.put(k, point(k, s.get(k)));
     return;
   }
+  if (st[0] != st[0]) {  // a line with a non-finite value (reduce_states): every point
+#pragma unroll 1
+    for (int k = 0; k < m; ++k) s.put(k, 0x7ff8000000000000ull);
+    return;
+  }
 #pragma unroll 1
   for (int k = 0; k < m; ++k) {
     uint64_t t[4], b;
