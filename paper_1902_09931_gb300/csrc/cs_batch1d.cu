@@ -374,6 +374,7 @@ __global__ void k_batch1d(const T* __restrict__ in, T* __restrict__ out,
 // Segments that hold infinities, NaN or only values outside 2^[-860, 870] take the FP64 chain.
 constexpr int kIxElems = 8;
 constexpr int kIxMinE = 160;  // with |c| >= 2^-100 no result is subnormal
+constexpr uint64_t kSumBias = 1ull << 63;  // |sum n_k X_k| <= 2^62, and rho's part below 2^19 more
 
 template <int L, int R>
 __global__ void __launch_bounds__(256, 3)
@@ -466,14 +467,14 @@ __global__ void __launch_bounds__(256, 3)
           sum[e] += __float2int_rn(c);
         }
       }
-      // sum c: the high 64 bits of the biased product, the bias's own share (cm is a multiple of 4) taken off
+      // sum c: the high 64 bits of the biased product, the bias's own share (cm is even) taken off
       const uint32_t ch = pn::hi32(ix.cm), cl = pn::lo32(ix.cm);
       const uint64_t ex = static_cast<uint64_t>(static_cast<uint32_t>(ix.ce + te - 1022 - ix.bits)) << 52;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const uint64_t u = static_cast<uint64_t>(sum[e]) + pn::kBias;
+        const uint64_t u = static_cast<uint64_t>(sum[e]) + kSumBias;
         const uint64_t lo = pn::wmul(pn::lo32(u), ch) + 0x80000000ull;
-        const uint64_t T = pn::wmul(pn::hi32(u), ch) + pn::hi32(lo) + pn::mad_hi(pn::hi32(u), cl, 0u) - (ix.cm >> 2);
+        const uint64_t T = pn::wmul(pn::hi32(u), ch) + pn::hi32(lo) + pn::mad_hi(pn::hi32(u), cl, 0u) - (ix.cm >> 1);
         const double x = __ll2double_rn(static_cast<long long>(T));
         res[e] = T ? pn::from_bits(pn::dbits(x) + ex) : 0.0;
       }

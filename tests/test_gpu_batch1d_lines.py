@@ -1,0 +1,70 @@
+"""Batched FP64 lines whose weights are c n_k (the fixed-point kernel): each output against its own five
+inputs' magnitude, so that lines of any scale may lie side by side."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+D2 = [-1 / 12, 16 / 12, -30 / 12, 16 / 12, -1 / 12]
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    import paper_1902_09931_gb300 as cs
+    cs.load()
+    return cs, torch
+
+
+def _run(env, x, off, w, left, right, bc):
+    cs, torch = env
+    d = torch.from_numpy(x).cuda()
+    out = torch.full_like(d, 5.0)
+    o = torch.from_numpy(off).cuda()
+    desc = cs.StencilDesc(dir=cs.CS_DIR_X, bc=bc, dtype=cs.CS_F64, left=left, right=right, weights=list(w))
+    plan = cs.cs_plan_create_1d_batch(desc, off.size - 1, o, x.size, d, out)
+    cs.cs_compute(plan)
+    torch.cuda.synchronize()
+    cs.cs_destroy(plan)
+    return out.cpu().numpy()
+
+
+def _reference(x, off, w, left, right, bc):
+    """(sums, sums of magnitudes) in extended precision; untouched outputs 5 and 0."""
+    ref, size = np.full(x.size, 5.0, dtype=np.longdouble), np.zeros(x.size, dtype=np.longdouble)
+    xl = x.astype(np.longdouble)
+    for a, b in zip(off[:-1], off[1:]):
+        n = b - a
+        if n == 0:
+            continue
+        k = np.arange(n)
+        t = [np.longdouble(w[p]) * xl[a + (k + p - left) % n] for p in range(left + right + 1)]
+        ok = np.ones(n, bool) if bc else (k >= left) & (k < n - right)
+        ref[a:b][ok], size[a:b][ok] = sum(t)[ok], sum(abs(v) for v in t)[ok]
+    return ref, size
+
+
+def _offsets(lengths):
+    return np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+
+
+# at most five roundings, each at most 2^-53 of a partial sum of the five products
+LIMIT = 5 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("w", [[1.0, -2.0, 1.0], [1.0, -2.0 * (1 + 2.0 ** -50), 1.0], [1.0, -2.0 - 2.0 ** -45, 1.0],
+                               [-1 / 12, 16 / 12, -30 / 12 * (1 + 2.0 ** -46), 16 / 12, -1 / 12], D2, [1.0, -1.0, 0.0], [3.0]])
+def test_values_just_below_a_power_of_two(env, w, sign):
+    """The weighted sum at the end of its range: values of the weights' signs (and their opposites) as near
+    to 1 as there are, with weights that are c n_k exactly and to 2^-45."""
+    r = len(w) // 2
+    s = np.sign(w)
+    s[s == 0] = 1.0
+    for top in (1 - 2.0 ** -53, 1 - 2.0 ** -48, 1 - 2.0 ** -21, 1 - 2.0 ** -20, 1.0):
+        x = sign * top * np.tile(s, 400)
+        off = _offsets([x.size])
+        ref, size = _reference(x, off, w, r, r, 1)
+        got = _run(env, x, off, w, r, r, 1)
+        assert (np.abs(got - ref) <= LIMIT * size).all(), (got[:6], ref[:6])
