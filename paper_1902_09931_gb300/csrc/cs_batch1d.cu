@@ -38,9 +38,11 @@ template <typename T> struct BTaps { T w[2 * CS_MAX_EXTENT + 1]; };
 // Weights as c (n_k + rho_k): integers n_k, sum |n_k| <= 64, |rho_k| small; c = cm 2^(ce - 64).
 struct IxLine {
   int32_t n[5];
-  float rho[5];  // in units of the fixed-point sum per 2^32 of the value
+  float size[5];  // |n_k|
+  float rho[5];   // in units of the fixed-point sum per 2^32 of the value
+  float need;     // least sum of |n_k X_k| / 2^32 of an output that fixed point may form
   int32_t ok, exact, ce;
-  int32_t bits;  // fixed-point bits of a value: the sum takes log2 of sum |n_k| more, 62 in all
+  int32_t bits;   // fixed-point bits of a value: the sum takes log2 of sum |n_k| more, 63 in all
   uint64_t cm;
 };
 
@@ -72,8 +74,13 @@ IxLine line_ratios(const Batch1DConfig* c) {
     }
     if (!fits) continue;
     ix.ok = ix.exact = 1;
-    ix.bits = 62;
+    ix.bits = 63;
     for (long long t = 1; t < total; t *= 2) --ix.bits;
+    // Fixed point cuts each X_k by less than one unit and rounds the sum and its product with c by less than
+    // six: at most 2^-52 of sum |n_k X_k| from (total + 6) 2^52 units on.  The kernel sums X_k's high words,
+    // each off by less than one, in FP32.
+    ix.need = static_cast<float>(((total + 6) * 1048576.0 + total) * (1.0 + 0x1p-20));
+    for (int i = 0; i < W; ++i) ix.size[i] = static_cast<float>(std::abs(ix.n[i]));
     int e;
     std::frexp(q, &e);  // q in [2^(e-1), 2^e)
     ix.cm = static_cast<uint64_t>(std::ldexp(q, 53 - e)) << 11;
@@ -361,20 +368,67 @@ __global__ void k_batch1d(const T* __restrict__ in, T* __restrict__ out,
                  static_cast<int64_t>(gridDim.x) * blockDim.x);
 }
 
+// The outputs of the lanes in `bad` (bit per lane of the segment at s) by the FMA chain, eight threads to a lane.
+// r0 .. r3 as for write_segment; outputs whose stencil leaves their line are not written.
+template <int L, int R, int E>
+__device__ __forceinline__ void chain_lanes(const double* __restrict__ in, double* __restrict__ out,
+                                            const int64_t* __restrict__ off, const int32_t* __restrict__ seg,
+                                            int64_t total, int64_t s, int r0, int r1, int r2, int r3, uint32_t bad,
+                                            const BTaps<double>& taps) {
+  static_assert(E == 8, "eight threads to a lane");
+  const int group = (threadIdx.x & 31) >> 3, e = threadIdx.x & 7;
+#pragma unroll 1
+  while (bad) {  // warp-uniform
+    int src = -1;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      if (group == g && bad) src = __ffs(static_cast<int>(bad)) - 1;
+      bad &= bad - 1;
+    }
+    const int o = src * E + e;
+    const int64_t k = s + o;
+    if (src < 0 || k >= total) continue;
+    int64_t ls, le;
+    if (o < r3) {
+      const int c = (o >= r1) + (o >= r2);
+      ls = s + (c == 0 ? r0 : (c == 1 ? r1 : r2));
+      le = s + (c == 0 ? r1 : (c == 1 ? r2 : r3));
+    } else {  // more lines in this segment than its four boundaries describe
+      int64_t m = __ldg(seg + (k >> kSegShift));
+      ls = __ldg(off + m);
+      le = __ldg(off + m + 1);
+      while (k >= le) {  // skips empty lines
+        ++m;
+        ls = le;
+        le = __ldg(off + m + 1);
+      }
+    }
+    if (k - ls < L || le - 1 - k < R) continue;
+    double acc = 0.0;
+#pragma unroll
+    for (int p = 0; p < L + R + 1; ++p) acc = fma(taps.w[p], __ldg(in + k - L + p), acc);
+    out[k] = acc;
+  }
+}
+
 // FP64 lines whose weights are c n_k with integers n_k, sum |n_k| <= 64, in 64-bit fixed point.  At two
 // FP64 instructions per clock and SM the five multiply-adds of a radius-2 stencil bound the FP64 walk at
-// 634 us for 63.5 M elements (FP32 storage 84 us; the floor of 16 bytes an element is 150 us).  Now 263 us,
-// bound by latency and the integer pipes (99 instructions an element).  Here a warp segment's
-// values become integers of 56 to 62 bits of its largest (62 with the bits that the sum takes), the
-// weighted sums are exact, and the one FP64 instruction left converts the scaled sum; what the weights miss of
-// c n_k joins the sum as an integer formed in FP32 (IxLine::rho), so the weights are the caller's to
-// 2^-60.  The result is the exact sum of the rounded inputs rounded twice, where the FMA chain rounds each
-// partial sum: error against 64-bit reference lines no larger (tests/test_gpu_batch1d_fixed.py).
-// 8 elements per lane, so that the two neighbours a lane of the segment's ends converts are shared by 8.
-// Segments that hold infinities, NaN or only values outside 2^[-860, 870] take the FP64 chain.
+// 634 us for 63.5 M elements (FP32 storage 84 us; the floor of 16 bytes an element is 150 us).  Here a
+// lane's window (8 elements and the neighbours that their stencils reach) becomes integers of 57 to 63 bits of
+// the window's largest value (63 with the bits that the sum takes), the weighted sums are exact, and the
+// one FP64 instruction left converts the scaled sum; what the weights miss of c n_k joins the sum as an
+// integer formed in FP32 (IxLine::rho), so the weights are the caller's to 2^-60.
+//
+// Each output keeps the accuracy of the FMA chain on its own inputs, whatever lies beside them: a lane
+// takes the chain (chain_lanes) unless, for every one of its outputs, sum |n_k X_k| is large enough that
+// the bits cut off the inputs stay below 2^-52 of it, and whenever its window reaches over the end of a line, so
+// that no line's values reach another's result.  8 elements per lane, so that the two neighbours on either side
+// are shared by 8.  In a smooth field with zeros and noise 2 % of the lanes take the chain, most of them at line
+// ends.  Lanes whose largest value is not finite, subnormal or outside 2^[-850, 870] take it too, and with inexact
+// weights those with a value within 2^-20 of the next power of two, where the sum could leave 63 bits.
 constexpr int kIxElems = 8;
-constexpr int kIxMinE = 160;  // with |c| >= 2^-100 no result is subnormal
-constexpr uint64_t kSumBias = 1ull << 63;  // |sum n_k X_k| <= 2^62, and rho's part below 2^19 more
+constexpr int kIxMinE = 173;  // with |c| >= 2^-100 no result is subnormal
+constexpr uint64_t kSumBias = 1ull << 63;
 
 template <int L, int R>
 __global__ void __launch_bounds__(256, 3)
@@ -419,88 +473,84 @@ __global__ void __launch_bounds__(256, 3)
   fetch(warp_id);
   for (int64_t sg = warp_id; sg < nseg; sg += nwarps) {  // warp-uniform loop
     const int64_t s = sg * kSeg, k0 = s + lane * E;
-    double v[E], h[H > 0 ? H : 1];
+    double v[E + 2 * H];  // the lane's window: v[H + e] its element e
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = nv[e];
+    for (int e = 0; e < E; ++e) v[H + e] = nv[e];
 #pragma unroll
-    for (int e = 0; e < H; ++e) h[e] = nh[e];
+    for (int e = 0; e < H; ++e) {
+      const double left = __shfl_up_sync(0xffffffffu, nv[E - H + e], 1), right = __shfl_down_sync(0xffffffffu, nv[e], 1);
+      v[e] = lane == 0 ? nh[e] : left;
+      v[H + E + e] = lane == 31 ? nh[e] : right;
+    }
     const int64_t m0 = nm0;
     const int64_t b = (lane < 4 && m0 + lane <= num_lines) ? __ldg(off + m0 + lane) : total;
     fetch(sg + nwarps);
-    uint32_t mx = 0;
+    uint32_t mx = 0, any = 0;
 #pragma unroll
-    for (int e = 0; e < E; ++e) mx = max(mx, pn::hi32(pn::dbits(v[e])) & 0x7fffffffu);
+    for (int e = 0; e < E + 2 * H; ++e) {
+      mx = max(mx, pn::hi32(pn::dbits(v[e])) & 0x7fffffffu);
+      any |= pn::lo32(pn::dbits(v[e]));
+    }
+    const int te = static_cast<int>(mx >> 20);
+    const bool zero = (mx | any) == 0u;  // every value zero
+    bool fixed = zero || (te >= kIxMinE && te <= pn::kMaxE && (ix.exact != 0 || (mx & 0xfffffu) != 0xfffffu));
+    const int sh = 64 - ix.bits + te;  // a zero window: at least 64 for its values, or mantissas of zero
+    int64_t win[E + 2 * H];
+    float f[E + 2 * H];
 #pragma unroll
-    for (int e = 0; e < H; ++e) mx = max(mx, pn::hi32(pn::dbits(h[e])) & 0x7fffffffu);
-    const int te = static_cast<int>(__reduce_max_sync(0xffffffffu, mx) >> 20);
+    for (int e = 0; e < E + 2 * H; ++e) {
+      win[e] = zero ? 0 : static_cast<int64_t>(pn::to_fixed(pn::dbits(v[e]), sh));
+      f[e] = __int2float_rn(static_cast<int>(win[e] >> 32));
+    }
+    float least = 3e38f;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      float size = 0.0f;
+#pragma unroll
+      for (int p = 0; p < W; ++p) size = fmaf(ix.size[p], fabsf(f[H - L + e + p]), size);
+      least = fminf(least, size);
+    }
+    fixed = fixed && (zero || least >= ix.need);
     double res[E];
-    if (te >= kIxMinE && te <= pn::kMaxE) {
-      const int sh = 64 - ix.bits + te;
-      int64_t win[E + 2 * H];
+    // sum c: the high 64 bits of the biased product, the bias's own share (cm is even) taken off
+    const uint32_t ch = pn::hi32(ix.cm), cl = pn::lo32(ix.cm);
+    const uint64_t ex = static_cast<uint64_t>(static_cast<uint32_t>(ix.ce + te - 1022 - ix.bits)) << 52;
 #pragma unroll
-      for (int e = 0; e < E; ++e) win[H + e] = static_cast<int64_t>(pn::to_fixed(pn::dbits(v[e]), sh));
+    for (int e = 0; e < E; ++e) {
+      int64_t sum = 0;
 #pragma unroll
-      for (int e = 0; e < H; ++e) {
-        const long long own = static_cast<long long>(pn::to_fixed(pn::dbits(h[e]), sh));
-        const long long left = __shfl_up_sync(0xffffffffu, static_cast<long long>(win[H + E - H + e]), 1);
-        const long long right = __shfl_down_sync(0xffffffffu, static_cast<long long>(win[H + e]), 1);
-        win[e] = lane == 0 ? own : left;
-        win[H + E + e] = lane == 31 ? own : right;
-      }
-      int64_t sum[E];
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        int64_t acc = 0;
-#pragma unroll
-        for (int p = 0; p < W; ++p) acc += ix.n[p] * win[H - L + e + p];
-        sum[e] = acc;
-      }
+      for (int p = 0; p < W; ++p) sum += ix.n[p] * win[H - L + e + p];
       if (ix.exact == 0) {
-        float f[E + 2 * H];
+        float c = 0.0f;
 #pragma unroll
-        for (int e = 0; e < E + 2 * H; ++e) f[e] = __int2float_rn(static_cast<int>(win[e] >> 32));
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          float c = 0.0f;
-#pragma unroll
-          for (int p = 0; p < W; ++p) c = fmaf(ix.rho[p], f[H - L + e + p], c);
-          sum[e] += __float2int_rn(c);
-        }
+        for (int p = 0; p < W; ++p) c = fmaf(ix.rho[p], f[H - L + e + p], c);
+        sum += __float2int_rn(c);
       }
-      // sum c: the high 64 bits of the biased product, the bias's own share (cm is even) taken off
-      const uint32_t ch = pn::hi32(ix.cm), cl = pn::lo32(ix.cm);
-      const uint64_t ex = static_cast<uint64_t>(static_cast<uint32_t>(ix.ce + te - 1022 - ix.bits)) << 52;
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const uint64_t u = static_cast<uint64_t>(sum[e]) + kSumBias;
-        const uint64_t lo = pn::wmul(pn::lo32(u), ch) + 0x80000000ull;
-        const uint64_t T = pn::wmul(pn::hi32(u), ch) + pn::hi32(lo) + pn::mad_hi(pn::hi32(u), cl, 0u) - (ix.cm >> 1);
-        const double x = __ll2double_rn(static_cast<long long>(T));
-        res[e] = T ? pn::from_bits(pn::dbits(x) + ex) : 0.0;
-      }
-    } else {
-      double win[E + 2 * H];
-#pragma unroll
-      for (int e = 0; e < E; ++e) win[H + e] = v[e];
-#pragma unroll
-      for (int e = 0; e < H; ++e) {
-        const double left = __shfl_up_sync(0xffffffffu, v[E - H + e], 1), right = __shfl_down_sync(0xffffffffu, v[e], 1);
-        win[e] = lane == 0 ? h[e] : left;
-        win[H + E + e] = lane == 31 ? h[e] : right;
-      }
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        double acc = 0.0;
-#pragma unroll
-        for (int p = 0; p < W; ++p) acc = fma(taps.w[p], win[H - L + e + p], acc);
-        res[e] = acc;
-      }
+      const uint64_t u = static_cast<uint64_t>(sum) + kSumBias;
+      const uint64_t lo = pn::wmul(pn::lo32(u), ch) + 0x80000000ull;
+      const uint64_t T = pn::wmul(pn::hi32(u), ch) + pn::hi32(lo) + pn::mad_hi(pn::hi32(u), cl, 0u) - (ix.cm >> 1);
+      const double x = __ll2double_rn(static_cast<long long>(T));
+      res[e] = T ? pn::from_bits(pn::dbits(x) + ex) : 0.0;
     }
     const int64_t d = b - s;
     const int r = static_cast<int>(d < -kClamp ? -kClamp : (d > kClamp ? kClamp : d));
     const int r0 = __shfl_sync(0xffffffffu, r, 0), r1 = __shfl_sync(0xffffffffu, r, 1);
     const int r2 = __shfl_sync(0xffffffffu, r, 2), r3 = __shfl_sync(0xffffffffu, r, 3);
-    if (k0 < total) write_segment<double, L, R, E>(out, off, total, vec_ok != 0, s, m0, r0, r1, r2, r3, res);
+    // a line boundary strictly inside the window, or boundaries beyond the segment's four
+    const int wl = lane * E - H, wr = lane * E + E + H;
+    auto inside = [&](int x) { return x > wl && x < wr; };
+    fixed = fixed && !inside(r0) && !inside(r1) && !inside(r2) && !inside(r3) && r3 > wl && k0 + E <= total;
+    if (fixed) {  // every output's stencil lies in one line
+      if (vec_ok) {
+#pragma unroll
+        for (int q = 0; q < E; q += 2) *reinterpret_cast<double2*>(out + k0 + q) = make_double2(res[q], res[q + 1]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) out[k0 + e] = res[e];
+      }
+    }
+    const uint32_t bad = __ballot_sync(0xffffffffu, !fixed && k0 < total);
+    if (bad) chain_lanes<L, R, E>(in, out, off, seg, total, s, r0, r1, r2, r3, bad, taps);
   }
   if (periodic && L + R > 0)
     line_ends<double>(in, out, off, num_lines, L, R, taps, static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x,

@@ -68,3 +68,43 @@ def test_values_just_below_a_power_of_two(env, w, sign):
         ref, size = _reference(x, off, w, r, r, 1)
         got = _run(env, x, off, w, r, r, 1)
         assert (np.abs(got - ref) <= LIMIT * size).all(), (got[:6], ref[:6])
+
+
+SCALES = [1.0, 1e-18, 1e20, 1e-8, 3e-100, 1.0, 1e150, 1e-12]
+
+
+@pytest.mark.parametrize("bc", [0, 1])
+@pytest.mark.parametrize("left, right, w", [(2, 2, D2), (2, 2, np.array(D2) * 1.7e7), (1, 1, [1.0, -2.0, 1.0]), (1, 2, [1.0, 3.0, -9.0, 2.0]),
+                                            (2, 0, [0.5, -2.0, 1.5]), (0, 0, [0.3])])
+def test_lines_of_different_scale_side_by_side(env, left, right, w, bc):
+    """Short and long lines of amplitudes 1e-100 to 1e150 packed next to one another, smooth and random, and
+    lines that decay over their length: every output to the bound of the multiply-add chain on its own inputs."""
+    rng = np.random.Generator(np.random.PCG64(left * 7 + right + bc))
+    off = _offsets(np.concatenate([rng.integers(1, 60, 200), [0, 256, 255, 0, 1, 8, 16, 300], rng.integers(64, 900, 60)]))
+    n = int(off[-1])
+    line = np.repeat(np.arange(off.size - 1), np.diff(off))
+    k = np.arange(n) - off[line]
+    scale = np.array(SCALES)[line % len(SCALES)]
+    decay = np.where(line % 3 == 0, np.exp2(-0.7 * np.minimum(k, 400)), 1.0)
+    for x in (scale * np.sin(0.1 * k + line), scale * rng.uniform(-1, 1, n), scale * decay * (1 + 0.3 * np.sin(0.05 * k)),
+              scale * np.where(rng.uniform(0, 1, n) < 0.7, 0.0, rng.uniform(-1, 1, n))):
+        ref, size = _reference(x, off, w, left, right, bc)
+        got = _run(env, x, off, w, left, right, bc)
+        assert (np.abs(got - ref) <= LIMIT * size).all(), float((np.abs(got - ref) / np.maximum(size, 1e-300)).max())
+
+
+def test_a_line_does_not_depend_on_its_neighbours(env):
+    """The same bits in a line whatever the other lines hold: other values, zeros, NaN."""
+    rng = np.random.Generator(np.random.PCG64(9))
+    off = _offsets(np.concatenate([rng.integers(1, 60, 100), rng.integers(200, 900, 30)]))
+    n = int(off[-1])
+    line = np.repeat(np.arange(off.size - 1), np.diff(off))
+    x = np.sin(0.07 * np.arange(n)) + 1e-3 * rng.uniform(-1, 1, n)
+    for w in (D2, [0.0, 1.0, -2.0, 1.0, 0.0], np.array(D2) * 0.37):
+        for bc in (0, 1):
+            ref = _run(env, x, off, w, 2, 2, bc)
+            for other in (1e20, 0.0, np.nan):
+                for keep in (0, 1):
+                    with np.errstate(invalid="ignore"):
+                        y = np.where(line % 2 == keep, x, other * x)
+                    assert np.array_equal(_run(env, y, off, w, 2, 2, bc)[line % 2 == keep], ref[line % 2 == keep])
