@@ -67,6 +67,7 @@ struct Par {
   uint64_t ic;               // 1 / c = ic 2^(ic_e - 62), ic in [2^61, 2^62)
   int ic_e;
   double eta, eps, inv_c;
+  double fs, bs;             // scales of the forward and backward states, the powers of two below 1 / sqrt(c) and 1 / c
   double M[4];               // A^m
   double Ml[6][4];           // A^(m 2^l): the scan's levels
   double R[4];               // backward state before a chunk caused by a unit forward state entering it
@@ -74,6 +75,7 @@ struct Par {
   double V[4];               // reflected: (W, E) after the line from (y, D) at its end
   double Z[4];               // reflected: the forward state entering the line from (W, E) at its start
   uint32_t low[4];           // mean low word of each table
+  uint32_t trunc_lo[4], trunc_hi[4];  // 2^31 times the share of points whose low / high word's product is truncated
   int t[4];                  // tables: real value = 2^t (int) / 2^60
 };
 
@@ -125,6 +127,20 @@ __host__ __device__ __forceinline__ uint64_t to_fixed(uint64_t xb, int E) {
   return (A ^ s) - s;
 }
 
+// to_fixed to the nearest integer, halves to the even one, on two more bits (E - (x's biased exponent) >= 2).
+// Cutting towards zero instead leaves half a unit of x's sign: harmless at a point, but the signs of a
+// slowly varying right-hand side stay, and their sum over a line is a drift of the conserved mass (4096^2,
+// 1000 steps: twice that of rounding each value).  The bits beyond the two are cut: 1/16 as much.
+__host__ __device__ __forceinline__ uint64_t to_fixed_near(uint64_t xb, int E) {
+  const uint32_t hi = hi32(xb);
+  const int e = static_cast<int>((hi >> 20) & 0x7ffu);
+  const uint64_t M = (static_cast<uint64_t>((hi & 0xFFFFFu) | 0x100000u) << 32 | lo32(xb)) << 11;
+  const uint64_t A4 = shr(M, E - 2 - e);
+  const uint64_t A = (A4 + (((lo32(A4) >> 2) & 1u) + 1u)) >> 2;
+  const uint64_t s = static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(hi) >> 31));
+  return (A ^ s) - s;
+}
+
 // T 2^e as a double, |T| < 2^62, rounded to nearest (halves away from zero: symmetric in sign).
 // The result must be a normal number or zero.
 __host__ __device__ __forceinline__ double from_fixed(uint64_t T, int e) {
@@ -158,8 +174,10 @@ __host__ __device__ __forceinline__ void step(uint64_t& Y, uint64_t& D, uint64_t
 
 // Phase 1 on one chunk, values at s (an accessor: load8 / store8 move 8 consecutive 64-bit words, get /
 // put one; the last m % 8 points are taken one by one).
-// Returns the scale mark: the exponent of W's unit, or kNative; ends = (y, D) / sqrt(c) after the
-// chunk and (W, E) / c before it.
+// Returns the scale mark: the exponent of W's unit, or kNative; ends = (y, D) after the chunk, about divided
+// by sqrt(c), and (W, E) before it, about divided by c.  The factors are powers of two, exact, and the
+// tables carry the rest: a rounded factor would leave an error in the line's sum that is the same at every
+// step for the slowly varying part of the field, a drift of the conserved mass.
 template <class Acc>
 __host__ __device__ __forceinline__ uint32_t chunk_max_hi(const Acc& s, int m) {
   uint32_t mx = 0;
@@ -191,37 +209,44 @@ __host__ __device__ __forceinline__ int local_fixed(const Par& q, const In& in, 
     in.load8(k0, v);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      step<WIDE>(Y, D, to_fixed(v[u], E), q.cn, q.ce, q.init_a, q.init_b, q.kc);
+      step<WIDE>(Y, D, to_fixed_near(v[u], E), q.cn, q.ce, q.init_a, q.init_b, q.kc);
       v[u] = Y;
     }
     s.store8(k0, v);
   }
   for (int k = m & ~7; k < m; ++k) {
-    step<WIDE>(Y, D, to_fixed(in.get(k), E), q.cn, q.ce, q.init_a, q.init_b, q.kc);
+    step<WIDE>(Y, D, to_fixed_near(in.get(k), E), q.cn, q.ce, q.init_a, q.init_b, q.kc);
     s.put(k, Y);
   }
-  ends[0] = static_cast<double>(static_cast<int64_t>(Y - kBias)) * (te ? q.eta * pow2(eu) : 0.0);
-  ends[1] = static_cast<double>(static_cast<int64_t>(D - kBias)) * (te ? q.eta * pow2(eu) : 0.0);
+  ends[0] = static_cast<double>(static_cast<int64_t>(Y - kBias)) * (te ? q.fs * pow2(eu) : 0.0);
+  ends[1] = static_cast<double>(static_cast<int64_t>(D - kBias)) * (te ? q.fs * pow2(eu) : 0.0);
   uint64_t W = kBias;
   D = kBias;
-  // from a zero state the first products are exact and make up for nothing: y is rounded there
-  s.put(m - 1, s.get(m - 1) + ((1ull << q.s2) >> 1));
-  for (int k = m - 1; k >= (m & ~7); --k) {
-    step<WIDE>(W, D, s.get(k) >> q.s2, q.cn, q.ce, q.init_a2, q.init_b, q.kc2);
-    s.put(k, W);
+  // y in W's unit.  init_a2 makes up for the mean of the bits that the shift drops, except at the chunk's
+  // two ends, where y is rounded to nearest even first: at the last point the products from a zero state
+  // are exact and make up for nothing, and y of the first point is b itself, whose bits below 2^-53
+  // are mostly zero (dropping them lost a quarter of W's unit instead of a half, a bias of 0.016 u a point of
+  // x at n = 512).  With wide coefficients D moves in steps of four, so y's low bits are b's at every point:
+  // all are rounded (0.23 u a point at n = 64 otherwise).
+  auto to_even = [&](uint64_t y) { return q.s2 ? y + ((1ull << (q.s2 - 1)) - 1 + ((y >> q.s2) & 1)) : y; };
+  if (!WIDE) {
+    s.put(m - 1, to_even(s.get(m - 1)));
+    s.put(0, to_even(s.get(0)));
   }
+  auto back = [&](uint64_t y, bool first) {
+    step<WIDE>(W, D, (WIDE ? to_even(y) : y) >> q.s2, q.cn, q.ce, WIDE || first ? q.init_a : q.init_a2, q.init_b, q.kc2);
+    return W;
+  };
+  for (int k = m - 1; k >= (m & ~7); --k) s.put(k, back(s.get(k), false));
   for (int k0 = (m & ~7) - 8; k0 >= 0; k0 -= 8) {
     uint64_t v[8];
     s.load8(k0, v);
 #pragma unroll
-    for (int u = 7; u >= 0; --u) {
-      step<WIDE>(W, D, v[u] >> q.s2, q.cn, q.ce, q.init_a2, q.init_b, q.kc2);
-      v[u] = W;
-    }
+    for (int u = 7; u >= 0; --u) v[u] = back(v[u], k0 + u == 0);
     s.store8(k0, v);
   }
-  ends[2] = static_cast<double>(static_cast<int64_t>(W - kBias)) * (te ? q.inv_c * pow2(eu + q.s2) : 0.0);
-  ends[3] = static_cast<double>(static_cast<int64_t>(D - kBias)) * (te ? q.inv_c * pow2(eu + q.s2) : 0.0);
+  ends[2] = static_cast<double>(static_cast<int64_t>(W - kBias)) * (te ? q.bs * pow2(eu + q.s2) : 0.0);
+  ends[3] = static_cast<double>(static_cast<int64_t>(D - kBias)) * (te ? q.bs * pow2(eu + q.s2) : 0.0);
   return te ? eu + q.s2 : -4000;
 }
 
@@ -246,8 +271,8 @@ __host__ __device__ __forceinline__ int local_native(const Par& q, const In& in,
     Y = Y + D;
     s.put(k, dbits(Y));
   }
-  ends[0] = Y * q.eta;
-  ends[1] = D * q.eta;
+  ends[0] = Y * q.fs;
+  ends[1] = D * q.fs;
   double W = 0.0;
   D = 0.0;
   for (int k = m - 1; k >= (m & ~7); --k) {
@@ -266,8 +291,8 @@ __host__ __device__ __forceinline__ int local_native(const Par& q, const In& in,
     }
     s.store8(k0, v);
   }
-  ends[2] = W * q.inv_c;
-  ends[3] = D * q.inv_c;
+  ends[2] = W * q.bs;
+  ends[3] = D * q.bs;
   return kNative;
 }
 
@@ -337,7 +362,9 @@ __host__ __device__ __forceinline__ bool corr_setup(const Par& q, int ew, const 
   // Rounding of the sum, in 2^-32 of an output unit: a truncated product is half a unit low on
   // average, a dropped low product lo lo / 2^64, with the table's mean low word over the chunk (a
   // statistical half instead would leave the chunk's sum, and with it the conserved mass, with a bias of
-  // a few hundredths of a unit a point); nothing when all is zero.
+  // a few hundredths of a unit a point); nothing when all is zero.  A product with a word that is the bias
+  // alone is exact: table values that have decayed below 2^-28 of the largest, at half of a chunk's points for
+  // small a, would otherwise be made up for too (up to 0.7 of a unit a point).
   uint64_t init = c.cw ? (1ull << 32) + (lo32(c.cw) >> 1) : 0ull;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -348,7 +375,9 @@ __host__ __device__ __forceinline__ bool corr_setup(const Par& q, int ew, const 
     const uint64_t sb = dbits(st[j]);
     const uint64_t v = bexp(st[j]) >= 64 ? (to_fixed(sb & 0x7fffffffffffffffull, E) + 8) & ~15ull : 0ull;
     c.u[j] = (static_cast<int64_t>(sb) < 0 ? 0ull - v : v) + kCoefBias;
-    if (c.u[j] != kCoefBias) init += (1ull << 32) + mad_hi(q.low[j], lo32(c.u[j]), 0u);
+    if (c.u[j] != kCoefBias)
+      init += static_cast<uint64_t>(q.trunc_hi[j]) + (hi32(c.u[j]) != hi32(kCoefBias) ? q.trunc_lo[j] : 0u) +
+              mad_hi(q.low[j], lo32(c.u[j]), 0u);
   }
   // bias terms that do not depend on k: W's bias times cw; the tables' bias times the states
   uint64_t k0 = c.cw >> 2;  // 2^62 cw / 2^64
@@ -461,6 +490,8 @@ inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<T
   q.eps = dd_val(eps);
   q.inv_c = dd_val(ic);
   q.wide = g.h <= 2.25;
+  q.fs = std::ldexp(1.0, std::ilogb(eta.h));
+  q.bs = std::ldexp(1.0, std::ilogb(ic.h));
   auto frac = [&](DD v) {  // v 2^64 (or 2^62), a multiple of 4; v <= 1 and < 0.8 when not wide
     const int k = q.wide ? 60 : 62;
     return static_cast<uint64_t>(dd_int(v, k)) << 2;
@@ -513,8 +544,7 @@ inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<T
   const uint64_t comp = (static_cast<uint64_t>(lo32(q.cn)) + lo32(q.ce)) >> 1;
   q.init_a = (1ull << 31) + (comp >> 1);
   q.init_b = (1ull << 31) + (comp >> 1);
-  const uint64_t down = (1ull << 31) - ((1ull << 31) >> q.s2);
-  q.init_a2 = q.init_a - (q.wide ? down >> 2 : down);
+  q.init_a2 = q.init_a - ((1ull << 31) - ((1ull << 31) >> q.s2));  // not used with wide coefficients
   {
     // the bias's own product, a whole number
     const uint64_t M = (q.cn >> 2) + (q.ce >> 2);
@@ -522,7 +552,8 @@ inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<T
     q.kc2 = q.kc - (kBias >> q.s2);
   }
   const M2 A{DD(1.0) - eta, DD(1.0) - eps, -eta, DD(1.0) - eps};
-  // homogeneous responses
+  // homogeneous responses, per unit of the scaled states
+  const DD icf = ic / DD(q.fs), icb = ic / DD(q.bs), bf(q.bs / q.fs);
   std::vector<DD> h[4];
   for (int j = 0; j < 4; ++j) h[j].resize(m);
   M2 Rr;
@@ -538,10 +569,10 @@ inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<T
     for (int k = m - 1; k >= 0; --k) {
       E = E + h[j][k] - (eta * W + eps * E);
       W = W + E;
-      h[j][k] = eta * W;
+      h[j][k] = icf * W;
     }
-    Rv[0][j] = eta * W;
-    Rv[1][j] = eta * E;
+    Rv[0][j] = bf * W;
+    Rv[1][j] = bf * E;
   }
   Rr = {Rv[0][0], Rv[0][1], Rv[1][0], Rv[1][1]};
   for (int j = 0; j < 2; ++j) {
@@ -549,7 +580,7 @@ inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<T
     for (int k = m - 1; k >= 0; --k) {
       E = E - (eta * W + eps * E);
       W = W + E;
-      h[2 + j][k] = W;
+      h[2 + j][k] = icb * W;
     }
   }
   tab.assign(m, TabRow{});
@@ -561,14 +592,21 @@ inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<T
     if (mx > 0.0) std::frexp(mx * (1.0 + 0x1p-40), &t);
     t = std::max(t, -900);
     q.t[j] = t;
-    uint64_t lows = 0;
+    uint64_t lows = 0, lo_used = 0, hi_used = 0;
+    DD left;  // what rounding the values so far left over, so that their sum is rounded only once
     for (int k = 0; k < m; ++k) {
-      const int64_t v = dd_int(h[j][k], 56 - t) * 16;  // whole sixteenths of 2^-60
+      const int64_t near = dd_int(h[j][k] + left, 56 - t);
+      left = h[j][k] + left - DD(std::ldexp(static_cast<double>(near >> 20), t - 36)) - DD(std::ldexp(static_cast<double>(near & 0xfffff), t - 56));
+      const int64_t v = near * 16;  // whole sixteenths of 2^-60
       tab[k].v[j] = static_cast<uint64_t>(v) + kCoefBias;
       base[k] -= tab[k].v[j] >> 4;
       lows += lo32(tab[k].v[j]);
+      lo_used += lo32(tab[k].v[j]) != 0;
+      hi_used += hi32(tab[k].v[j]) != hi32(kCoefBias);
     }
     q.low[j] = static_cast<uint32_t>(lows / m);
+    q.trunc_lo[j] = static_cast<uint32_t>((lo_used << 31) / m);
+    q.trunc_hi[j] = static_cast<uint32_t>((hi_used << 31) / m);
   }
   put(Rr, q.R);
   M2 Am{DD(1.0), DD(), DD(), DD(1.0)}, sq = A;
@@ -605,7 +643,8 @@ inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<T
     put(inv(sub_from_id(pw[P])), q.C);
   } else {
     // mirrored ends: (W, E) after the line = V (y, D) there; (y, D) before it = Q (W, E) at its start
-    const M2 V{DD(1.0), qq / eps, DD(), eta / eps}, Q{DD(1.0), -(qq / eta), DD(), eps / eta};
+    const DD vs = bf / eta, qs = eta / bf;
+    const M2 V{vs, qq / eps * vs, DD(), bf / eps}, Q{qs, -(qq / bf), DD(), eps / bf};
     put(V, q.V);
     M2 N = add(mul(Rr, pw[P - 1]), mul(Am, mul(V, pw[P])));
     for (int p = P - 1;; --p) {
