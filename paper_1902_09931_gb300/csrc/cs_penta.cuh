@@ -302,6 +302,10 @@ __host__ __device__ __forceinline__ int local_solve(const Par& q, const In& in, 
                                                     double (&ends)[4]) {
   const uint32_t mx = chunk_max_hi(in, m);
   const int te = static_cast<int>(mx >> 20);
+  if (te == 0x7ff) {  // a non-finite value: the whole line is filled from its end values (correct_chunk)
+    ends[0] = ends[1] = ends[2] = ends[3] = from_bits(0x7ff8000000000000ull);
+    return kNative;
+  }
   if (q.native || (te != 0 && (te < kMinE || te > kMaxE))) return local_native(q, in, s, m, ends);
   return q.wide ? local_fixed<1>(q, in, s, m, te, ends) : local_fixed<0>(q, in, s, m, te, ends);
 }
