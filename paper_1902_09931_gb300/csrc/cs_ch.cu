@@ -1048,9 +1048,12 @@ __global__ void __launch_bounds__(kSolveThreads)
   correct_chunk(q, TabGlobal(lt), s, m, scale[pl * lines + line], st);
 }
 
-// Valid partition: P divides n, chunks of at least 16 points in whole register batches.
+// Valid partition: P divides n, chunks of at least 16 points, in whole register batches or (the solves
+// take the last m % 8 points one by one) any power of two of them on the grids of 64 points' multiples.
+bool whole_batches(int64_t n, int P) { return P >= 1 && n % P == 0 && (n / P) % kU == 0; }
 bool valid_chunks(int64_t n, int P) {
-  return P >= 1 && P <= 64 && n % P == 0 && (n / P) >= 16 && (n / P) % kU == 0;
+  return P >= 1 && P <= pn::kMaxChunks && n % P == 0 && n / P >= 16 &&
+         (whole_batches(n, P) || (n % 64 == 0 && (P & (P - 1)) == 0));
 }
 
 // Chunks of at least 16 points up to 32 chunks a line, of at least 32 beyond: the threads of a line
@@ -1061,7 +1064,7 @@ bool valid_chunks(int64_t n, int P) {
 int default_chunks(int64_t n) {
   auto longest = [&](bool any) {
     int P = 1;
-    while (2 * P <= pn::kMaxChunks && n % (2 * P) == 0 && (any || valid_chunks(n, 2 * P)) &&
+    while (2 * P <= pn::kMaxChunks && n % (2 * P) == 0 && (any || whole_batches(n, 2 * P)) &&
            n / (2 * P) >= (P < 32 ? 16 : 32))
       P *= 2;
     return P;
@@ -1708,7 +1711,7 @@ int set_partition(CHPlan* p, int P) {
 
 }  // namespace
 
-// Times one step for every valid chunk count (1 .. 64 chunks per line) from the plan's current
+// Times one step for the plan's chunk count and every power of two (1 .. 64 chunks per line) from the plan's current
 // state, keeps the fastest, records it in the tuning table, and restores the fields.
 int ch_autotune(CHPlan* p, cudaStream_t s) {
   const size_t eb = p->storage == CS_F32 ? 4 : 8;
@@ -1727,8 +1730,10 @@ int ch_autotune(CHPlan* p, cudaStream_t s) {
   int rc = e == cudaSuccess ? CS_OK : cuda_error(e, "autotune setup");
   int best = p->P;
   float best_ms = 1e30f;
-  for (int P = 1; P <= 64 && rc == CS_OK; P *= 2) {
-    if (!valid_chunks(p->n, P)) continue;
+  const int first = p->P;  // the plan's own partition first: another has to beat it
+  for (int c = 0; c <= 7 && rc == CS_OK; ++c) {
+    const int P = c == 0 ? first : 1 << (c - 1);
+    if (!valid_chunks(p->n, P) || (c > 0 && P == first)) continue;
     rc = set_partition(p, P);
     if (rc != CS_OK) break;
     rc = ch_step(p, 1, nullptr, nullptr, s);  // warm-up
