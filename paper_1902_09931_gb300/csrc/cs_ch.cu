@@ -651,6 +651,27 @@ struct AccStride {  // words es apart (shared or global memory)
   __device__ __forceinline__ uint64_t get(int k) const { return p[k * es]; }
   __device__ __forceinline__ void put(int k, uint64_t v) const { p[k * es] = v; }
 };
+// 32-byte global accesses: a whole sector per thread and instruction
+__device__ __forceinline__ void ld_words4(const uint64_t* p, uint64_t& a, uint64_t& b, uint64_t& c, uint64_t& d) {
+  asm volatile("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_words4(uint64_t* p, uint64_t a, uint64_t b, uint64_t c, uint64_t d) {
+  asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+}
+struct AccWide {  // words in a row of global memory, 32-byte aligned
+  uint64_t* p;
+  int64_t es;
+  __device__ __forceinline__ void load8(int k, uint64_t (&v)[8]) const {
+    ld_words4(p + k, v[0], v[1], v[2], v[3]);
+    ld_words4(p + k + 4, v[4], v[5], v[6], v[7]);
+  }
+  __device__ __forceinline__ void store8(int k, const uint64_t (&v)[8]) const {
+    st_words4(p + k, v[0], v[1], v[2], v[3]);
+    st_words4(p + k + 4, v[4], v[5], v[6], v[7]);
+  }
+  __device__ __forceinline__ uint64_t get(int k) const { return p[k]; }
+  __device__ __forceinline__ void put(int k, uint64_t v) const { p[k] = v; }
+};
 template <int ES>
 struct AccCols {  // ES columns interleaved (shared memory)
   uint64_t* p;
@@ -970,6 +991,8 @@ __global__ void __launch_bounds__(256)
 // Lines too long for shared memory, and the columns of a row band (whose chunks lie on several ranks):
 // the two phases as kernels over global memory, one thread per (line, chunk), with the same
 // functions, so the same values.  G holds W, scale the chunks' scale marks.
+// Acc: AccWide for rows whose chunks are 32-byte aligned, else AccStride.
+template <class Acc>
 __global__ void __launch_bounds__(kSolveThreads)
     k_line_local(const double* __restrict__ in, uint64_t* __restrict__ G, double* __restrict__ bnd,
                  int* __restrict__ scale, const pn::Par q, int64_t lines, int Pl, int m, int64_t line_stride,
@@ -978,8 +1001,8 @@ __global__ void __launch_bounds__(kSolveThreads)
   if (t >= lines * Pl) return;
   const int64_t line = t % lines, pl = t / lines;
   const int64_t at = line * line_stride + pl * m * elem_stride;
-  const AccStride si{const_cast<uint64_t*>(reinterpret_cast<const uint64_t*>(in)) + at, elem_stride};
-  AccStride s{G + at, elem_stride};
+  const Acc si{const_cast<uint64_t*>(reinterpret_cast<const uint64_t*>(in)) + at, elem_stride};
+  const Acc s{G + at, elem_stride};
   double ends[4];
   scale[pl * lines + line] = pn::local_solve(q, si, s, m, ends);
 #pragma unroll
@@ -1002,18 +1025,24 @@ __global__ void __launch_bounds__(8 * pn::kMaxChunks)
     for (int j = 0; j < 4; ++j) states[(4 * static_cast<int64_t>(p) + j) * lines + line] = st[j];
 }
 
-template <int MODE, typename T>
+template <int MODE, typename T, bool WIDE>
 struct AccOut {  // reads W, writes the result of phase 2
   const uint64_t* p;
   double* out;
   T* next;
   int64_t es;
   __device__ __forceinline__ void load8(int k, uint64_t (&v)[8]) const {
+    if constexpr (WIDE) {
+      AccWide{const_cast<uint64_t*>(p), 1}.load8(k, v);
+    } else {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = p[(k + u) * es];
+      for (int u = 0; u < 8; ++u) v[u] = p[(k + u) * es];
+    }
   }
   __device__ __forceinline__ void store8(int k, const uint64_t (&v)[8]) const {
-    if constexpr (MODE == 0) {
+    if constexpr (MODE == 0 && WIDE) {
+      AccWide{reinterpret_cast<uint64_t*>(out), 1}.store8(k, v);
+    } else if constexpr (MODE == 0) {
 #pragma unroll
       for (int u = 0; u < 8; ++u) out[(k + u) * es] = pn::from_bits(v[u]);
     } else {
@@ -1032,7 +1061,7 @@ struct AccOut {  // reads W, writes the result of phase 2
 };
 
 // MODE 0 writes x (FP64) to out; MODE 1 adds it to Cbar in next.
-template <int MODE, typename T>
+template <int MODE, typename T, bool WIDE = false>
 __global__ void __launch_bounds__(kSolveThreads)
     k_line_correct(uint64_t* __restrict__ G, const double* __restrict__ states, const int* __restrict__ scale,
                    const pn::Par q, const LineTab lt, int64_t lines, int p0, int Pl, int m, int64_t line_stride,
@@ -1041,7 +1070,7 @@ __global__ void __launch_bounds__(kSolveThreads)
   if (t >= lines * Pl) return;
   const int64_t line = t % lines, pl = t / lines;
   const int64_t at = line * line_stride + pl * m * elem_stride;
-  AccOut<MODE, T> s{G + at, MODE == 0 ? out + at : nullptr, MODE == 1 ? next + at : nullptr, elem_stride};
+  AccOut<MODE, T, WIDE> s{G + at, MODE == 0 ? out + at : nullptr, MODE == 1 ? next + at : nullptr, elem_stride};
   double st[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) st[j] = states[(4 * (p0 + pl) + j) * lines + line];
@@ -1201,12 +1230,15 @@ int launch_rows(const Lines& L, bool noflux, int64_t rows, const double* in, dou
     return CS_OK;
   }
   const unsigned grid = static_cast<unsigned>((rows * P + kSolveThreads - 1) / kSolveThreads);
-  k_line_local<<<grid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(B), line_ends(L), line_scale(L, rows), L.par,
-                                              rows, P, m, n, 1);
+  uint64_t* G = reinterpret_cast<uint64_t*>(B);
+  // every chunk of a row (n is a multiple of 64) starts on a 32-byte boundary
+  const bool wide = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(B)) & 31u) == 0 && m % 4 == 0;
+  auto local = wide ? k_line_local<AccWide> : k_line_local<AccStride>;
+  auto correct = wide ? k_line_correct<0, double, true> : k_line_correct<0, double, false>;
+  local<<<grid, kSolveThreads, 0, s>>>(in, G, line_ends(L), line_scale(L, rows), L.par, rows, P, m, n, 1);
   launch_states(L, noflux, rows, line_ends(L), s);
-  k_line_correct<0, double><<<grid, kSolveThreads, 0, s>>>(reinterpret_cast<uint64_t*>(B), line_states(L, rows),
-                                                           line_scale(L, rows), L.par, lt, rows, 0, P, m, n, 1, out,
-                                                           static_cast<double*>(nullptr));
+  correct<<<grid, kSolveThreads, 0, s>>>(G, line_states(L, rows), line_scale(L, rows), L.par, lt, rows, 0, P, m, n, 1, out,
+                                         static_cast<double*>(nullptr));
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(3);
   return CS_OK;
@@ -1238,7 +1270,7 @@ int launch_cols(const Lines& L, bool noflux, const double* in, T* next, double* 
     return CS_OK;
   }
   const unsigned grid = static_cast<unsigned>((n * P + kSolveThreads - 1) / kSolveThreads);
-  k_line_local<<<grid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(B), line_ends(L), line_scale(L, n), L.par, n, P,
+  k_line_local<AccStride><<<grid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(B), line_ends(L), line_scale(L, n), L.par, n, P,
                                               m, 1, n);
   launch_states(L, noflux, n, line_ends(L), s);
   k_line_correct<1, T><<<grid, kSolveThreads, 0, s>>>(reinterpret_cast<uint64_t*>(B), line_states(L, n), line_scale(L, n),
@@ -1949,7 +1981,7 @@ int ch_band_ycols_local(CHBand* b, int64_t chunk0, const double* in, double* end
   if (rc != CS_OK) return rc;
   const int Pl = static_cast<int>(b->rows / b->m);
   const unsigned sgrid = static_cast<unsigned>((b->n * Pl + kSolveThreads - 1) / kSolveThreads);
-  k_line_local<<<sgrid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(b->B), ends, line_scale(b->lines, b->n),
+  k_line_local<AccStride><<<sgrid, kSolveThreads, 0, s>>>(in, reinterpret_cast<uint64_t*>(b->B), ends, line_scale(b->lines, b->n),
                                                b->lines.par, b->n, Pl, b->m, 1, b->n);
   CS_CUDA_TRY(cudaGetLastError());
   count_launches(1);
