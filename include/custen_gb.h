@@ -222,8 +222,9 @@ int cs_plan_set_fp64_mode(cs_plan_t plan, int32_t mode);
  *   2  TMA-pipelined persistent sweep: tiles of 64 rows, each CTA walks its tiles through a
  *      two-stage shared-memory ring filled by tensor-memory-access copies (used when nx is a
  *      multiple of 16 bytes / element size and d_in is 16-byte aligned, else 1).
- * A plan for which neither the caller nor the autotuner chose reports 2 here, runs in groups with
- * 64-row tiles, and runs alone with the shape that its type, size and alignment call for.
+ * A plan for which neither the caller nor the autotuner chose reports 2 here, and runs, alone or in
+ * a group, with CTAs of the height that its type, size and alignment call for; its FP64 integer-digit
+ * results are those of choices 1 and 2 whatever that height is.
  * Choices 1 and 2 give the same results bit for bit (the same tiles).  Choice 0 does too for
  * FP32 storage; on the FP64 integer-digit path its digit grid is set by 32-row tiles, so results
  * can differ from choices 1 and 2 within that path's error bound.  CS_EINVAL for another value. */

@@ -129,7 +129,7 @@ __device__ __forceinline__ void load_tile_interior(T* s, const T* __restrict__ i
 template <typename T, bool COMPACT = false>
 __device__ __forceinline__ void load_tile(T* s, const T* __restrict__ in, int64_t nx, int64_t ny,
                                           bool periodic, bool vec_ok, int64_t x0, int64_t y0,
-                                          int top, int LA, int cols, int rows) {
+                                          int top, int LA, int cols, int rows, int beyond = 0) {
   constexpr int V = Vec<T>::n;
   const int nch = cols / V;
   const int total = rows * nch;
@@ -155,7 +155,8 @@ __device__ __forceinline__ void load_tile(T* s, const T* __restrict__ in, int64_
   // Any other tile.  Where rows are 16-byte aligned (nx a multiple of V; the tile's columns start at
   // one) a 16-byte chunk lies inside the grid or outside it as a whole, so it wraps as a chunk; else
   // element by element, without the wraps where the tile lies inside the grid.
-  const bool one_wrap = nx >= cols && ny >= rows;  // tile halo reaches at most one period out
+  // the tile and its halo reach at most one period out (a tile may start `beyond` rows past the grid's last tile)
+  const bool one_wrap = nx >= cols && ny >= rows + beyond;
   auto wrapped = [&](int64_t k, int64_t n) { return one_wrap ? (k < 0 ? k + n : (k >= n ? k - n : k)) : wrap_idx(k, n); };
   if constexpr (COMPACT) {
 #pragma unroll 1
@@ -232,13 +233,13 @@ __device__ __forceinline__ void load_tile(T* s, const T* __restrict__ in, int64_
 template <typename T, int ROWS, int COLS, bool COMPACT = false>
 __device__ __forceinline__ void load_tile_ct(T* s, const T* __restrict__ in, int64_t nx, int64_t ny,
                                              bool periodic, bool vec_ok, int64_t x0, int64_t y0,
-                                             int top, int LA) {
+                                             int top, int LA, int beyond = 0) {
   const int64_t gy0 = y0 - top, gx0 = x0 - LA;
   if (vec_ok && gy0 >= 0 && gy0 + ROWS <= ny && gx0 >= 0 && gx0 + COLS <= nx) {
     load_tile_interior<T, ROWS, COLS>(s, in, nx, gy0, gx0);
     return;
   }
-  load_tile<T, COMPACT>(s, in, nx, ny, periodic, vec_ok, x0, y0, top, LA, COLS, ROWS);
+  load_tile<T, COMPACT>(s, in, nx, ny, periodic, vec_ok, x0, y0, top, LA, COLS, ROWS, beyond);
 }
 
 template <typename T>
@@ -699,6 +700,26 @@ __device__ __forceinline__ void ix_compute(const int2* sd2, double* __restrict__
   }
 }
 
+// Pairs: two CTAs of a cluster take the 32-row halves of one 64-row tile and share its largest exponent, so the
+// digit grid (and the choice of the native path) is the 64-row tile's, and so is every bit of the result.
+constexpr int kPairRows = 64;
+__device__ __forceinline__ void pair_start() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+// The larger of both CTAs' v (uniform over each); slot: a word of shared memory.  Waits for pair_start of both,
+// so that the peer is there to be written to; after the second barrier nobody touches the peer's memory.
+__device__ __forceinline__ unsigned pair_max(unsigned v, unsigned* slot) {
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (threadIdx.x == 0) {
+    unsigned rank, addr;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(addr) : "r"(static_cast<unsigned>(__cvta_generic_to_shared(slot))), "r"(rank ^ 1u));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+  return max(v, *static_cast<volatile unsigned*>(slot));
+}
+
 // Resident CTAs of the digit kernel: at least 6 (40 registers per thread, 48 warps per SM; the
 // tile's shared memory allows 6) for footprints of at most 13 taps over at most 5 rows, whose
 // rolling digit sums fit that budget; at least 3 (85 registers) for the larger footprints.  More
@@ -713,7 +734,7 @@ template <int TY, int SPEC, bool FULL, int CW = 0>
 __global__ void __launch_bounds__(kThreads, ix_min_blocks(SPEC))
     k_stencil2d_ix(const double* __restrict__ in, double* __restrict__ out, int64_t nx, int64_t ny,
                    int periodic, int vec_ok, Taps<double> taps, IxTaps itaps, int tx0, int ty0, int ring_nbx,
-                   int ring_nby) {
+                   int ring_nby, int pair) {
   constexpr SpecDesc sd = kSpecs[SPEC];
   constexpr int V = Vec<double>::n;
   constexpr int TX = tile_x<double>();
@@ -723,10 +744,13 @@ __global__ void __launch_bounds__(kThreads, ix_min_blocks(SPEC))
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* s = reinterpret_cast<double*>(smem_raw);
   __shared__ __align__(16) unsigned s_red[kThreads / 32];
+  __shared__ unsigned s_pair;
   static_assert(COLS % 2 == 0, "digit passes take values in pairs");
+  constexpr bool kMayPair = 2 * TY == kPairRows;
+  if (kMayPair && pair) pair_start();
   // the tile: (blockIdx.x + tx0, blockIdx.y + ty0), or with ring_nbx > 0 the CTA's tile of the
   // border ring of an nbx x nby tile grid (the top row, the bottom row, then the first and last
-  // columns of the rows between)
+  // columns of the rows between; of pairs, blockIdx.y the half)
   int64_t bx = static_cast<int64_t>(blockIdx.x) + tx0, by = static_cast<int64_t>(blockIdx.y) + ty0;
   if (ring_nbx > 0) {
     const int b = static_cast<int>(blockIdx.x), mid = ring_nby - 2;
@@ -741,14 +765,17 @@ __global__ void __launch_bounds__(kThreads, ix_min_blocks(SPEC))
       bx = side ? ring_nbx - 1 : 0;
       by = 1 + (c - side * mid);
     }
+    if (kMayPair && pair) by = 2 * by + blockIdx.y;
   }
   const int64_t x0 = bx * TX;
   const int64_t y0 = by * TY;
   overlap_wait();
-  load_tile_ct<double, ROWS, COLS, FULL>(s, in, nx, ny, periodic != 0, vec_ok != 0, x0, y0, sd.T, LA);
+  load_tile_ct<double, ROWS, COLS, FULL>(s, in, nx, ny, periodic != 0, vec_ok != 0, x0, y0, sd.T, LA,
+                                         kMayPair && pair ? TY : 0);
   // pass 1: the tile's largest exponent; inf / nan (and tiles outside the exponent window) take
   // native FP64
-  const uint32_t mhi = ixd::ix_tile_max_hi<kThreads, ROWS * COLS>(s, s_red);
+  uint32_t mhi = ixd::ix_tile_max_hi<kThreads, ROWS * COLS>(s, s_red);
+  if (kMayPair && pair) mhi = pair_max(mhi, &s_pair);
   const int tile_e = static_cast<int>(mhi >> 20);
   uint32_t w[4];
   if (!ixi_consts(itaps.c, itaps.c15, tile_e, w) || (sd.epi && !ixf_tile_ok(tile_e, itaps.c))) {
@@ -778,9 +805,32 @@ inline void window_tiles(int ty, int64_t ny, int* ty0, int* nty) {
   *nty = static_cast<int>(t1 > t0 ? t1 - t0 : 0);
 }
 
+// Launches a tile kernel of kThreads, over the previous kernel's tail where `overlap` says so, in
+// clusters of K CTAs along y.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_tiles(void (*kern)(KArgs...), dim3 grid, size_t smem, cudaStream_t st, bool overlap, int K,
+                                Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  if (overlap) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (K > 1) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs++].val.clusterDim = {1, static_cast<unsigned>(K), 1};
+  }
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 template <int TY, int SPEC>
 int launch_ix(const double* in, double* out, int64_t nx, int64_t ny, int periodic, int vec_ok,
-              const Taps<double>& taps, const IxTaps& itaps, const Stencil2DConfig* cfg, cudaStream_t st) {
+              const Taps<double>& taps, const IxTaps& itaps, const Stencil2DConfig* cfg, int pair, cudaStream_t st) {
   constexpr SpecDesc sd = kSpecs[SPEC];
   constexpr int TX = tile_x<double>();
   const size_t smem = tile_smem_bytes<double>(sd.L, sd.R, sd.T, sd.B, TY, false);
@@ -794,17 +844,19 @@ int launch_ix(const double* in, double* out, int64_t nx, int64_t ny, int periodi
     CS_CUDA_TRY(cudaFuncSetAttribute(kedge, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
     attr_set = true;
   }
+  // tiles of TP rows, of K CTAs each (pairs: the 64-row tile's two halves)
+  const int K = pair ? kPairRows / TY : 1, TP = K * TY;
   int ty0, nty;
-  window_tiles(TY, ny, &ty0, &nty);
+  window_tiles(TP, ny, &ty0, &nty);
   if (nty == 0) return CS_OK;
-  const int64_t nbx = (nx + TX - 1) / TX, nby = (ny + TY - 1) / TY;
+  const int64_t nbx = (nx + TX - 1) / TX, nby = (ny + TP - 1) / TP;
   // the FULL form (every output of a tile written, 16-byte stores) applies to every tile of a
   // periodic grid of whole tiles, and to the inner tiles of a non-periodic one
-  const bool whole = nx % TX == 0 && ny % TY == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  const bool whole = nx % TX == 0 && ny % TP == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   if (periodic || !whole || !cfg || !cfg->aux || ty0 != 0 || nty != nby || nbx < 3 || nby < 3) {
     auto kern = periodic && whole ? kfull : kedge;
-    dim3 grid(static_cast<unsigned>(nbx), static_cast<unsigned>(nty));
-    CS_CUDA_TRY(launch_overlapped(kern, grid, dim3(kThreads), smem, st, in, out, nx, ny, periodic, vec_ok, taps, itaps, 0, ty0, 0, 0));
+    dim3 grid(static_cast<unsigned>(nbx), static_cast<unsigned>(K * nty));
+    CS_CUDA_TRY(launch_tiles(kern, grid, smem, st, true, K, in, out, nx, ny, periodic, vec_ok, taps, itaps, 0, K * ty0, 0, 0, pair));
     CS_CUDA_TRY(cudaGetLastError());
     count_launches(1);
     return CS_OK;
@@ -814,12 +866,12 @@ int launch_ix(const double* in, double* out, int64_t nx, int64_t ny, int periodi
   CS_CUDA_TRY(cudaEventRecord(cfg->ev_fork, st));
   CS_CUDA_TRY(cudaStreamWaitEvent(cfg->aux, cfg->ev_fork, 0));
   const unsigned nring = static_cast<unsigned>(2 * nbx + 2 * (nby - 2));
-  kedge<<<nring, kThreads, smem, cfg->aux>>>(in, out, nx, ny, periodic, vec_ok, taps, itaps, 0, 0,
-                                             static_cast<int>(nbx), static_cast<int>(nby));
+  CS_CUDA_TRY(launch_tiles(kedge, dim3(nring, static_cast<unsigned>(K)), smem, cfg->aux, false, K, in, out, nx, ny, periodic,
+                           vec_ok, taps, itaps, 0, 0, static_cast<int>(nbx), static_cast<int>(nby), pair));
   CS_CUDA_TRY(cudaGetLastError());
   CS_CUDA_TRY(cudaEventRecord(cfg->ev_join, cfg->aux));
-  dim3 grid(static_cast<unsigned>(nbx - 2), static_cast<unsigned>(nby - 2));
-  kfull<<<grid, kThreads, smem, st>>>(in, out, nx, ny, periodic, vec_ok, taps, itaps, 1, 1, 0, 0);
+  dim3 grid(static_cast<unsigned>(nbx - 2), static_cast<unsigned>(K * (nby - 2)));
+  CS_CUDA_TRY(launch_tiles(kfull, grid, smem, st, false, K, in, out, nx, ny, periodic, vec_ok, taps, itaps, 1, K, 0, 0, pair));
   CS_CUDA_TRY(cudaGetLastError());
   CS_CUDA_TRY(cudaStreamWaitEvent(st, cfg->ev_join, 0));
   count_launches(2);
@@ -829,10 +881,10 @@ int launch_ix(const double* in, double* out, int64_t nx, int64_t ny, int periodi
 template <int TY>
 int dispatch_ix(int variant, const double* in, double* out, int64_t nx, int64_t ny, int periodic,
                 int vec_ok, const Taps<double>& taps, const IxTaps& itaps, const Stencil2DConfig* cfg,
-                cudaStream_t st) {
+                int pair, cudaStream_t st) {
   switch (variant) {
 #define CS_IX_CASE(I) \
-  case I: return launch_ix<TY, I>(in, out, nx, ny, periodic, vec_ok, taps, itaps, cfg, st);
+  case I: return launch_ix<TY, I>(in, out, nx, ny, periodic, vec_ok, taps, itaps, cfg, pair, st);
     CS_IX_CASE(0) CS_IX_CASE(1) CS_IX_CASE(2) CS_IX_CASE(3) CS_IX_CASE(4)
     CS_IX_CASE(5) CS_IX_CASE(6) CS_IX_CASE(7) CS_IX_CASE(8) CS_IX_CASE(9)
     CS_IX_CASE(10) CS_IX_CASE(11) CS_IX_CASE(13)
@@ -1576,25 +1628,32 @@ int make_tensor_map(const Stencil2DConfig* cfg, const void* in, int elem_bytes, 
 
 // The tile shape a sweep runs with: the plan's own where the caller or the autotuner chose one, else
 // by size (times on GB300, back to back, us; the same bits for FP32 storage whatever the shape, and for
-// FP64 storage between 64-row tiles and TMA):
-//   FP64 storage on the digit or double-float path: tiles of 32 rows up to 2^22.5 points, where more
-//   CTAs hide each other's load and reduction phases (9-point Laplacian, 256^2 3.8 against 5.4 with 64
-//   rows and 5.7 with TMA; 2048^2 18.2 / 19.8 / 20.9; 3072^2 34.9 / 34.6 / 38.5), 64 rows beyond
-//   (4096^2 57.6 / 54.6 / 61.4; 8192^2 biharmonic 230 / 201 / 240), and 32 rows for rows that are not
-//   16-byte aligned (4097^2 69.0 / 77.2);
+// FP64 storage between 64-row tiles, TMA and pairs):
+//   FP64 storage on the digit path: 64-row tiles (9-point Laplacian, 1024^2 6.6 against 7.9 with 32 rows, 2048^2
+//   15.5 / 15.8, 4096^2 53.3 / 56.9; 8192^2 biharmonic 201, TMA 240), in pairs of CTAs where the tiles are
+//   fewer than the SMs (256^2 4.1 against 4.9; 1024^2 8.9 against 6.6).  32-row tiles would take 3.4 at 256^2 and
+//   68 against 76 at 4097^2, but on a digit grid of their own: a plan alone, the same plan in a group
+//   and a band of its grid would differ in the last bits;
+//   FP64 storage on the double-float path: 32 rows up to 2^22.5 points and for rows that are not 16-byte
+//   aligned (d2x8 4097 x 2049 55.4 against 59.9), where more CTAs hide each other's load and reduction phases;
 //   FP32 storage: 32 rows (512^2 2.7 / 3.5 / 4.0; 4096^2 23.7 / 24.1 / 24.3; 8192^2 84.5 / 84.0 /
 //   94.8; 4097^2 32.1 / 38.3), except TMA for non-periodic stencils that reach sideways on 2^20 to
 //   2^23 points (2048^2 7.6 / 7.4 / 7.1).
-struct TileShape { int rows; bool tma; };
+struct TileShape { int rows; bool tma, pair; };
 template <typename T> TileShape tile_shape(const Stencil2DConfig* cfg) {
-  if (!cfg->auto_shape || cfg->variant < 0) return {cfg->tile_rows, cfg->use_tma != 0};
+  if (!cfg->auto_shape || cfg->variant < 0) return {cfg->tile_rows, cfg->use_tma != 0, false};
   const int64_t cells = cfg->cells;
   if (sizeof(T) == 8) {
-    if (cfg->fp64_mode != CS_FP64_AUTO || !(cfg->ix_ok || cfg->dd_ok)) return {cfg->tile_rows, cfg->use_tma != 0};
-    return {cells <= 5931641 || cfg->nx % 2 != 0 ? 32 : 64, false};
+    if (cfg->fp64_mode != CS_FP64_AUTO || !(cfg->ix_ok || cfg->dd_ok)) return {cfg->tile_rows, cfg->use_tma != 0, false};
+    if (cfg->ix_ok) {
+      const int64_t tiles = (cfg->nx + tile_x<double>() - 1) / tile_x<double>() * ((cfg->ny + kPairRows - 1) / kPairRows);
+      const bool pair = tiles <= num_sms();
+      return {pair ? 32 : 64, false, pair};
+    }
+    return {cells <= 5931641 || cfg->nx % 2 != 0 ? 32 : 64, false, false};
   }
   const bool tma = cfg->bc != CS_BC_PERIODIC && cfg->left + cfg->right > 0 && cells > (1 << 20) && cells <= (1 << 23);
-  return {tma ? 64 : 32, tma};
+  return {tma ? 64 : 32, tma, false};
 }
 
 template <typename T>
@@ -1657,8 +1716,8 @@ int launch_stencil2d_t(const Stencil2DConfig* cfg, const void* vin, void* vout, 
         it.inv_hi = static_cast<float>(1.0 / cfg->ix_c);
         it.inv_lo = static_cast<float>(1.0 / cfg->ix_c - static_cast<double>(it.inv_hi));
         if (shape.rows == 32)
-          return dispatch_ix<32>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, it, cfg, st);
-        return dispatch_ix<64>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, it, cfg, st);
+          return dispatch_ix<32>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, it, cfg, shape.pair, st);
+        return dispatch_ix<64>(cfg->variant, in, out, cfg->nx, cfg->ny, periodic, vec_ok, taps, it, cfg, 0, st);
       }
       if (cfg->dd_ok && cfg->fp64_mode == CS_FP64_AUTO) {
         DDTaps dt;
