@@ -731,8 +731,9 @@ int cs_autotune(cs_plan_t p, void* stream) {
   if (p->kind == kCahnHilliard) return ch_autotune(p->ch, static_cast<cudaStream_t>(stream));
   if (p->kind == kStencil2DHost || p->kind == kWeno) return CS_OK;  // one launch shape: nothing to choose
   if (p->elems == 0) return CS_OK;
+  const int nchoices = p->kind == kStencil2D ? stencil2d_num_tile_choices() : batch1d_num_choices(&p->b1);
+  if (nchoices == 1) return CS_OK;  // nor here; the tuning key is that of plans with other weights too
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int nchoices = p->kind == kStencil2D ? stencil2d_num_tile_choices() : batch1d_num_choices();
   cudaEvent_t e0, e1;
   CS_CUDA_TRY(cudaEventCreate(&e0));
   CS_CUDA_TRY(cudaEventCreate(&e1));

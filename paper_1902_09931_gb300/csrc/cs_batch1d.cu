@@ -35,17 +35,6 @@ template <> struct Vec1<double> { static constexpr int n = 2; using V = double2;
 
 template <typename T> struct BTaps { T w[2 * CS_MAX_EXTENT + 1]; };
 
-// Weights as c (n_k + rho_k): integers n_k, sum |n_k| <= 64, |rho_k| small; c = cm 2^(ce - 64).
-struct IxLine {
-  int32_t n[5];
-  float size[5];  // |n_k|
-  float rho[5];   // in units of the fixed-point sum per 2^32 of the value
-  float need;     // least sum of |n_k X_k| / 2^32 of an output that fixed point may form
-  int32_t ok, exact, ce;
-  int32_t bits;   // fixed-point bits of a value: the sum takes log2 of sum |n_k| more, 63 in all
-  uint64_t cm;
-};
-
 // The fixed-point form of a radius-2 stencil's weights, ok = 0 when they have none (no common scale to
 // 2^-44 of the largest weight, as the 2D sweeps' digit path asks, or one outside 2^[-100, 100]).
 IxLine line_ratios(const Batch1DConfig* c) {
@@ -581,6 +570,20 @@ int launch_t(const Batch1DConfig* c, const void* vin, void* vout, cudaStream_t s
   const int W = c->left + c->right + 1;
   for (int i = 0; i < 2 * CS_MAX_EXTENT + 1; ++i)
     taps.w[i] = i < W ? static_cast<T>(c->weights[i]) : T(0);
+  const int vec_ok = (reinterpret_cast<uintptr_t>(in) % 16 == 0) && (reinterpret_cast<uintptr_t>(out) % 16 == 0);
+  if constexpr (sizeof(T) == 8 && LL >= 0) {
+    if (c->ix.ok) {
+      int fit = 0;
+      CS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_batch1d_ix<LL, RR>, 256, 0));
+      const int64_t nseg = (c->total_len + 32 * kIxElems - 1) / (32 * kIxElems);
+      const int64_t grid = std::min<int64_t>((nseg + 7) / 8, static_cast<int64_t>(num_sms()) * std::max(fit, 1));
+      CS_CUDA_TRY(launch_overlapped(k_batch1d_ix<LL, RR>, dim3(static_cast<unsigned>(std::max<int64_t>(grid, 1))), dim3(256),
+                                    0, st, in, out, c->d_offsets, c->d_seg_line, c->total_len, c->num_lines,
+                                    c->bc == CS_BC_PERIODIC, vec_ok, taps, c->ix));
+      count_launches(1);
+      return CS_OK;
+    }
+  }
   const LaunchShape sh = kShapes[c->choice];
   const bool generic = LL < 0;
   auto kern = generic ? k_batch1d_generic<T> : nullptr;
@@ -601,22 +604,6 @@ int launch_t(const Batch1DConfig* c, const void* vin, void* vout, cudaStream_t s
         in, out, c->d_offsets, c->d_seg_line, c->total_len, c->num_lines, c->bc == CS_BC_PERIODIC,
         c->left, c->right, taps));
   } else {
-    const int vec_ok = (reinterpret_cast<uintptr_t>(in) % 16 == 0) &&
-                       (reinterpret_cast<uintptr_t>(out) % 16 == 0);
-    if constexpr (sizeof(T) == 8) {
-      const IxLine ix = line_ratios(c);
-      if (ix.ok) {
-        int fit = 0;
-        CS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_batch1d_ix<LL, RR>, 256, 0));
-        const int64_t nseg = (c->total_len + 32 * kIxElems - 1) / (32 * kIxElems);
-        const int64_t grid = std::min<int64_t>((nseg + 7) / 8, static_cast<int64_t>(num_sms()) * std::max(fit, 1));
-        CS_CUDA_TRY(launch_overlapped(k_batch1d_ix<LL, RR>, dim3(static_cast<unsigned>(std::max<int64_t>(grid, 1))), dim3(256),
-                                      0, st, in, out, c->d_offsets, c->d_seg_line, c->total_len, c->num_lines,
-                                      c->bc == CS_BC_PERIODIC, vec_ok, taps, ix));
-        count_launches(1);
-        return CS_OK;
-      }
-    }
     const int64_t seg_elems = 32 * lane_elems<T>();
     const int64_t nseg = (c->total_len + seg_elems - 1) / seg_elems;
     const int64_t warps_per_cta = sh.threads / 32;
@@ -653,6 +640,7 @@ int batch1d_prepare(Batch1DConfig* c, cudaStream_t st) {
   c->d_seg_line = nullptr;
   c->num_table = 0;
   c->choice = 1;
+  c->ix = line_ratios(c);
   if (c->total_len == 0) return CS_OK;
   c->num_table = ((c->total_len - 1) >> kSegShift) + 1;
   CS_CUDA_TRY(cudaMalloc(&c->d_seg_line, c->num_table * sizeof(int32_t)));
@@ -672,7 +660,7 @@ void batch1d_release(Batch1DConfig* c) {
   c->d_seg_line = nullptr;
 }
 
-int batch1d_num_choices() { return kNumShapes; }
+int batch1d_num_choices(const Batch1DConfig* c) { return c->ix.ok ? 1 : kNumShapes; }
 
 std::string batch1d_shape_key(const Batch1DConfig* c) {
   char buf[160];
@@ -797,6 +785,7 @@ extern "C" int cs_batch1d_compute_noalloc(const cs_stencil_desc* d, int64_t num_
   c.left = d->left;
   c.right = d->right;
   for (int i = 0; i < d->left + d->right + 1; ++i) c.weights[i] = d->weights[i];
+  c.ix = line_ratios(&c);
   c.d_offsets = d_offsets;
   c.d_seg_line = scratch;
   c.num_table = ((total_len - 1) >> kSegShift) + 1;

@@ -107,6 +107,16 @@ int stencil2d_group(const Stencil2DConfig* const* cfgs, const void* const* ins, 
 constexpr int kMaxGroupJobs = 64;
 
 // ---- batched 1D (cs_batch1d.cu) -------------------------------------------------------------
+// A radius-2 stencil's weights as c (n_k + rho_k): integers n_k, sum |n_k| <= 64, |rho_k| small; c = cm 2^(ce - 64).
+struct IxLine {
+  int32_t n[5];
+  float size[5];  // |n_k|
+  float rho[5];   // in units of the fixed-point sum per 2^32 of the value
+  float need;     // least sum of |n_k X_k| / 2^32 of an output that fixed point may form
+  int32_t ok, exact, ce;
+  int32_t bits;   // fixed-point bits of a value: the sum takes log2 of sum |n_k| more, 63 in all
+  uint64_t cm;
+};
 struct Batch1DConfig {
   int64_t num_lines, total_len;
   int bc, dtype, left, right;
@@ -115,11 +125,12 @@ struct Batch1DConfig {
   int32_t* d_seg_line;       // library-owned: line containing element s * kSegTable
   int64_t num_table;
   int choice;                // launch shape index
+  IxLine ix;                 // from the weights, when the plan is made
 };
 int batch1d_prepare(Batch1DConfig* cfg, cudaStream_t s);
 void batch1d_release(Batch1DConfig* cfg);
 int batch1d_launch(const Batch1DConfig* cfg, const void* in, void* out, cudaStream_t s);
-int batch1d_num_choices();
+int batch1d_num_choices(const Batch1DConfig* cfg);  // 1: the fixed-point kernel has one launch shape
 std::string batch1d_shape_key(const Batch1DConfig* cfg);
 
 // ---- periodic XY WENO advection (cs_weno.cu) ---------------------------------------------------

@@ -108,3 +108,18 @@ def test_a_line_does_not_depend_on_its_neighbours(env):
                     with np.errstate(invalid="ignore"):
                         y = np.where(line % 2 == keep, x, other * x)
                     assert np.array_equal(_run(env, y, off, w, 2, 2, bc)[line % 2 == keep], ref[line % 2 == keep])
+
+
+def test_nothing_to_tune_in_fixed_point(env):
+    """The fixed-point kernel has one launch shape: the autotuner launches nothing for it and leaves the
+    tuning key, which plans with other weights share, alone."""
+    cs, torch = env
+    off = torch.arange(0, 6401, 64, device="cuda")
+    x = torch.rand(6400, device="cuda", dtype=torch.float64)
+    out = torch.zeros_like(x)
+    for w, tuned in ((D2, False), ([0.1, 0.7, -1.3, 0.9, 0.25], True)):
+        plan = cs.cs_plan_create_1d_batch(cs.StencilDesc(dir=cs.CS_DIR_X, bc=1, dtype=cs.CS_F64, left=2, right=2, weights=w), 100, off, 6400, x, out)
+        before = cs.cs_launch_count()
+        cs.cs_autotune(plan)
+        assert (cs.cs_launch_count() > before) == tuned
+        cs.cs_destroy(plan)
