@@ -1102,6 +1102,15 @@ int default_chunks(int64_t n) {
   return n / P <= 64 ? P : longest(true);
 }
 
+// Tuning key of the partition.  Not the former solver's "ch|...": its best chunk counts (16 at 4096^2), saved in a
+// file, would keep this one from its own.
+std::string partition_key(int storage, bool noflux, int64_t n) {
+  char key[96];
+  snprintf(key, sizeof key, "chlines|%s%s|n%lld|sm%d", storage == CS_F32 ? "f32" : "f64", noflux ? "|noflux" : "",
+           (long long)n, num_sms());
+  return key;
+}
+
 // FP64 tiles (C^n, Cbar: halo 2; Z: halo 1), for either storage type.
 size_t rhs_smem_bytes() {
   return 8 * (2 * (kTY + 4) * (kTX + 4));  // C^n and Cbar (Z reuses Cbar's space)
@@ -1373,10 +1382,7 @@ int ch_create(CHPlan** out, const cs_ch_desc* d, void* prev, void* cur, void* ne
   p->alpha = (2.0 / 3.0) * d->D * d->dt / h2;
   int P = default_chunks(d->n);
   int choice;
-  char key[96];
-  snprintf(key, sizeof key, "ch|%s%s|n%lld|sm%d", d->storage == CS_F32 ? "f32" : "f64",
-           p->noflux ? "|noflux" : "", (long long)d->n, num_sms());
-  if (tune_lookup(key, &choice) && valid_chunks(d->n, choice)) P = choice;
+  if (tune_lookup(partition_key(d->storage, p->noflux, d->n), &choice) && valid_chunks(d->n, choice)) P = choice;
   p->P = P;
   p->m = static_cast<int>(d->n / P);
   p->field[0] = prev; p->field[1] = cur; p->field[2] = next;
@@ -1790,10 +1796,7 @@ int ch_autotune(CHPlan* p, cudaStream_t s) {
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (rc != CS_OK) return rc;
-  char key[96];
-  snprintf(key, sizeof key, "ch|%s%s|n%lld|sm%d", p->storage == CS_F32 ? "f32" : "f64",
-           p->noflux ? "|noflux" : "", (long long)p->n, num_sms());
-  tune_store(key, best);
+  tune_store(partition_key(p->storage, p->noflux, p->n), best);
   return CS_OK;
 }
 
@@ -1872,10 +1875,7 @@ void free_band(CHBand* b) {
 // for it when one is recorded, else the default.
 static int band_partition(const cs_ch_desc* d) {
   int P = default_chunks(d->n), choice;
-  char key[96];
-  snprintf(key, sizeof key, "ch|%s%s|n%lld|sm%d", d->storage == CS_F32 ? "f32" : "f64",
-           d->boundary == CS_CH_NOFLUX ? "|noflux" : "", (long long)d->n, num_sms());
-  if (tune_lookup(key, &choice) && valid_chunks(d->n, choice)) P = choice;
+  if (tune_lookup(partition_key(d->storage, d->boundary == CS_CH_NOFLUX, d->n), &choice) && valid_chunks(d->n, choice)) P = choice;
   return P;
 }
 

@@ -17,3 +17,19 @@ def test_default_partition_is_replayed(cs, boundary, n):
     assert P * m == n
     for a in (0.7, 2885.8, 1.85e5):
         assert cs.cs_ch_solver_check(n, P, a, boundary) <= 64 * 2.0 ** -52  # the bound of every other partition
+
+
+def test_tune_files_of_the_former_solver_are_not_read(tmp_path):
+    """Its chunk counts (16 at 4096^2) are not this solver's; what the autotuner saves now is (own process:
+    the tuning table is process-wide)."""
+    import subprocess
+    import sys
+    old, new = tmp_path / "old.json", tmp_path / "new.json"
+    keys = [f"{{}}|f64|n4096|sm{sms}" for sms in (148, 152, 160)]
+    old.write_text("{" + ", ".join(f'"{k.format("ch")}": 16' for k in keys) + "}")
+    new.write_text("{" + ", ".join(f'"{k.format("chlines")}": 32' for k in keys) + "}")
+    code = ("import sys, paper_1902_09931_gb300 as cs; cs.load(); d = cs.CHDesc(n=4096, storage=0, D=1.0, gamma=0.01, dt=0.01)\n"
+            "print(cs.cs_ch_partition(d)[0]); cs.cs_tune_load(sys.argv[1]); print(cs.cs_ch_partition(d)[0])\n"
+            "cs.cs_tune_load(sys.argv[2]); print(cs.cs_ch_partition(d)[0])")
+    got = subprocess.run([sys.executable, "-c", code, str(old), str(new)], capture_output=True, text=True, check=True).stdout.split()
+    assert got == ["64", "64", "32"]
