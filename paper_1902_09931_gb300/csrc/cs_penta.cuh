@@ -250,7 +250,8 @@ __host__ __device__ __forceinline__ int local_fixed(const Par& q, const In& in, 
   return te ? eu + q.s2 : -4000;
 }
 
-// The same in FP64, for chunks outside fixed point's exponents (infinities and NaN go through it).
+// The same in FP64, for chunks outside fixed point's exponents, on y fs and W bs: W itself is up to c times the
+// result and would overflow first.
 template <class In, class Acc>
 __host__ __device__ __forceinline__ int local_native(const Par& q, const In& in, const Acc& s, int m,
                                                      double (&ends)[4]) {
@@ -260,23 +261,24 @@ __host__ __device__ __forceinline__ int local_native(const Par& q, const In& in,
     in.load8(k0, v);
 #pragma unroll 1
     for (int u = 0; u < 8; ++u) {
-      D = D + (from_bits(v[u]) - fma(q.eta, Y, q.eps * D));
+      D = D + (from_bits(v[u]) * q.fs - fma(q.eta, Y, q.eps * D));
       Y = Y + D;
       v[u] = dbits(Y);
     }
     s.store8(k0, v);
   }
   for (int k = m & ~7; k < m; ++k) {
-    D = D + (from_bits(in.get(k)) - fma(q.eta, Y, q.eps * D));
+    D = D + (from_bits(in.get(k)) * q.fs - fma(q.eta, Y, q.eps * D));
     Y = Y + D;
     s.put(k, dbits(Y));
   }
-  ends[0] = Y * q.fs;
-  ends[1] = D * q.fs;
+  ends[0] = Y;
+  ends[1] = D;
+  const double to_w = q.bs / q.fs;  // a power of two
   double W = 0.0;
   D = 0.0;
   for (int k = m - 1; k >= (m & ~7); --k) {
-    D = D + (from_bits(s.get(k)) - fma(q.eta, W, q.eps * D));
+    D = D + (from_bits(s.get(k)) * to_w - fma(q.eta, W, q.eps * D));
     W = W + D;
     s.put(k, dbits(W));
   }
@@ -285,14 +287,14 @@ __host__ __device__ __forceinline__ int local_native(const Par& q, const In& in,
     s.load8(k0, v);
 #pragma unroll 1
     for (int u = 7; u >= 0; --u) {
-      D = D + (from_bits(v[u]) - fma(q.eta, W, q.eps * D));
+      D = D + (from_bits(v[u]) * to_w - fma(q.eta, W, q.eps * D));
       W = W + D;
       v[u] = dbits(W);
     }
     s.store8(k0, v);
   }
-  ends[2] = W * q.bs;
-  ends[3] = D * q.bs;
+  ends[2] = W;
+  ends[3] = D;
   return kNative;
 }
 
@@ -410,7 +412,7 @@ __host__ __device__ __forceinline__ uint64_t corr_point(const Corr& c, uint64_t 
 // x at point k of a chunk in FP64 (the chunk's W at scale mark ew)
 __host__ __device__ __forceinline__ double corr_native(const Par& q, int ew, uint64_t W, const uint64_t* t,
                                                        const double (&st)[4]) {
-  double x = ew == kNative ? from_bits(W) * q.inv_c
+  double x = ew == kNative ? from_bits(W) * (q.inv_c / q.bs)
              : ew > -4000  ? static_cast<double>(static_cast<int64_t>(W - kBias)) * pow2(ew) * q.inv_c
                            : 0.0;
 #pragma unroll
@@ -479,13 +481,16 @@ inline void put(const M2& x, double* o) {
 // Constants and tables of lines of n points in P chunks, for the coefficient a.  tab: m rows; base: m;
 // mats: 8 doubles per chunk, A^(m (p + 1)) and (reflected lines) the response of the backward state
 // before chunk p to a unit forward state entering the line.  False when the constants leave the
-// representable range (a not finite or above 1e300).
+// representable range (a not finite).
 inline bool build(int64_t n, int P, double a, bool noflux, Par& q, std::vector<TabRow>& tab,
                   std::vector<uint64_t>& base, std::vector<double>& mats) {
   memset(&q, 0, sizeof q);
-  if (!(a >= 0.0) || !(a <= 1e300)) return false;
+  if (!(a >= 0.0) || !std::isfinite(a)) return false;
   q.native = a > 1e24;
   const int m = static_cast<int>(n / P);
+  // beyond 1e40 a line of 65536 points or less is its mean to 2^-70, and the constants' last digits would be lost
+  // in 1 - A^n
+  a = std::min(a, 1e40);
   const DD r = dd_sqrt(DD(1.0) + DD(16.0) * DD(a));
   const DD g = dd_sqrt((DD(1.0) + r) * DD(0.5));
   const DD eta = DD(2.0) / (g * (g + DD(1.0))), eps = DD(2.0) / (g + DD(1.0)), qq = DD(1.0) - eps;

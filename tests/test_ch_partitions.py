@@ -33,3 +33,10 @@ def test_tune_files_of_the_former_solver_are_not_read(tmp_path):
             "cs.cs_tune_load(sys.argv[2]); print(cs.cs_ch_partition(d)[0])")
     got = subprocess.run([sys.executable, "-c", code, str(old), str(new)], capture_output=True, text=True, check=True).stdout.split()
     assert got == ["64", "64", "32"]
+
+
+@pytest.mark.parametrize("boundary", [0, 1])
+@pytest.mark.parametrize("a", [1e24, 1e25, 1e60, 1e200, 1e300, 1e301, 1e304, 1e307, 1.7e308])
+def test_every_finite_coefficient(cs, a, boundary):
+    for n, P in ((64, 1), (64, 4), (1024, 32)):
+        assert cs.cs_ch_solver_check(n, P, a, boundary) <= 64 * 2.0 ** -52
