@@ -266,9 +266,9 @@ def cs_compute(plan, stream=None) -> None:
 
 def cs_compute_group(plans, stream=None) -> None:
     """One grouped launch (per 64 plans) over several 2D stencil plans of the same shape."""
-    try:
-        arr = b"".join(plans)  # the handles' own bytes: c_void_p objects are buffers
-    except TypeError:  # plain addresses among them
+    if set(map(type, plans)) == {ctypes.c_void_p}:
+        arr = b"".join(plans)  # the handles' own bytes (other buffers must not pass for handles)
+    else:  # plain addresses among them
         arr = (ctypes.c_void_p * len(plans))(*[p.value if hasattr(p, "value") else p for p in plans])
     _check((_lib or load()).cs_compute_group(arr, len(plans), _stream(stream)))
 
