@@ -483,12 +483,12 @@ __global__ void __launch_bounds__(256, 3)
     const int te = static_cast<int>(mx >> 20);
     const bool zero = (mx | any) == 0u;  // every value zero
     bool fixed = zero || (te >= kIxMinE && te <= pn::kMaxE && (ix.exact != 0 || (mx & 0xfffffu) != 0xfffffu));
-    const int sh = 64 - ix.bits + te;  // a zero window: at least 64 for its values, or mantissas of zero
+    const int sh = zero ? 4096 : 64 - ix.bits + te;  // to_fixed shifts everything out of a zero window
     int64_t win[E + 2 * H];
     float f[E + 2 * H];
 #pragma unroll
     for (int e = 0; e < E + 2 * H; ++e) {
-      win[e] = zero ? 0 : static_cast<int64_t>(pn::to_fixed(pn::dbits(v[e]), sh));
+      win[e] = static_cast<int64_t>(pn::to_fixed(pn::dbits(v[e]), sh));
       f[e] = __int2float_rn(static_cast<int>(win[e] >> 32));
     }
     float least = 3e38f;
