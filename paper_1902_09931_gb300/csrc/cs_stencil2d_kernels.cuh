@@ -1630,10 +1630,10 @@ int make_tensor_map(const Stencil2DConfig* cfg, const void* in, int elem_bytes, 
 // by size (times on GB300, back to back, us; the same bits for FP32 storage whatever the shape, and for
 // FP64 storage between 64-row tiles, TMA and pairs):
 //   FP64 storage on the digit path: 64-row tiles (9-point Laplacian, 1024^2 6.6 against 7.9 with 32 rows, 2048^2
-//   15.5 / 15.8, 4096^2 53.3 / 56.9; 8192^2 biharmonic 201, TMA 240), in pairs of CTAs where the tiles are
-//   fewer than the SMs (256^2 4.1 against 4.9; 1024^2 8.9 against 6.6).  32-row tiles would take 3.4 at 256^2 and
-//   68 against 76 at 4097^2, but on a digit grid of their own: a plan alone, the same plan in a group
-//   and a band of its grid would differ in the last bits;
+//   15.5 / 15.8, 4096^2 53.3 / 56.9; 8192^2 biharmonic 201, TMA 240), in pairs of CTAs up to three CTAs per SM
+//   (256^2 4.1 against 4.9, 896^2 5.6 / 6.7; 1024^2 8.9 / 6.6).
+//   32-row tiles would take 3.4 at 256^2 and 68 against 76 at 4097^2, but on a digit grid of their own: a plan
+//   alone, the same plan in a group and a band of its grid would differ in the last bits;
 //   FP64 storage on the double-float path: 32 rows up to 2^22.5 points and for rows that are not 16-byte
 //   aligned (d2x8 4097 x 2049 55.4 against 59.9), where more CTAs hide each other's load and reduction phases;
 //   FP32 storage: 32 rows (512^2 2.7 / 3.5 / 4.0; 4096^2 23.7 / 24.1 / 24.3; 8192^2 84.5 / 84.0 /
@@ -1647,7 +1647,7 @@ template <typename T> TileShape tile_shape(const Stencil2DConfig* cfg) {
     if (cfg->fp64_mode != CS_FP64_AUTO || !(cfg->ix_ok || cfg->dd_ok)) return {cfg->tile_rows, cfg->use_tma != 0, false};
     if (cfg->ix_ok) {
       const int64_t tiles = (cfg->nx + tile_x<double>() - 1) / tile_x<double>() * ((cfg->ny + kPairRows - 1) / kPairRows);
-      const bool pair = tiles <= num_sms();
+      const bool pair = 2 * tiles <= 3 * num_sms();
       return {pair ? 32 : 64, false, pair};
     }
     return {cells <= 5931641 || cfg->nx % 2 != 0 ? 32 : 64, false, false};
