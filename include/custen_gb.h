@@ -54,8 +54,8 @@ typedef enum { CS_DIR_X = 0, CS_DIR_Y = 1, CS_DIR_XY = 2 } cs_dir;
  * (cells with i < left, i >= nx - right, j < top, j >= ny - bottom; Sec. 3 and Sec. 4.1). */
 typedef enum { CS_BC_NONPERIODIC = 0, CS_BC_PERIODIC = 1 } cs_bc;
 
-/* Storage (and stencil arithmetic) type of the fields.  CS_F32 stencils compute in FP32;
- * Cahn-Hilliard line solves and reductions always run in FP64. */
+/* Storage (and stencil arithmetic) type of the fields.  CS_F32 stencils compute in FP32; the
+ * Cahn-Hilliard step computes on widened values at FP64's precision whatever the storage. */
 typedef enum { CS_F64 = 0, CS_F32 = 1 } cs_dtype;
 
 /* The "Fun" variant (Sec. 4.2, Sec. 5.2).  The paper takes a user device-function pointer
@@ -111,7 +111,10 @@ int cs_plan_create_2d(cs_plan_t* plan, const cs_stencil_desc* desc, const void* 
 
 /* Create for a ragged batch of 1D lines (Abstract; Sec. 5.4's batched 1D problems): line m
  * occupies elements [offsets[m], offsets[m+1]) of the packed buffers.  desc->dir must be
- * CS_DIR_X (top = bottom = 0); a periodic stencil wraps at each line's own length.
+ * CS_DIR_X (top = bottom = 0); a periodic stencil wraps at each line's own length.  Lines are
+ * independent: a line's result does not depend on the values of the others.  CS_F64: every output is
+ * within five roundings of its own products, 5 * 2^-53 of sum_p |w_p x_p|, for stencils of up to
+ * two points on either side.
  *   d_offsets  device array of num_lines + 1 int64 values, non-decreasing, offsets[0] = 0,
  *              offsets[num_lines] = total_len, every line shorter than 2^31 elements.  Read at create time (the library builds its
  *              load-balancing table from it) and by every compute; must stay alive.
@@ -279,7 +282,8 @@ int cs_destroy(cs_plan_t plan);
  * uses the coefficient of L_x, the reading under which steady states of the scheme are steady
  * states of the equation.
  *   n        grid points per side (n x n), a multiple of 64 in [64, 65536]
- *   storage  CS_F64, or CS_F32 (fields stored in FP32, stencils in FP32, solves in FP64)
+ *   storage  CS_F64, or CS_F32 (fields stored in FP32 and widened; the right-hand side in integer
+ *            digits, the line solves in 64-bit fixed point or FP64, reductions in FP64)
  *   D, gamma mobility and interface parameter (Sec. 5.3: 1.0 and 0.01)
  *   dt       time step (Sec. 5.3: 0.1 h)
  *   boundary CS_CH_PERIODIC (0, the paper's case) or CS_CH_NOFLUX: the same scheme on a
@@ -412,8 +416,9 @@ int cs_ch_band_ycols_correct(cs_plan_t plan, int64_t chunk0, const double* d_end
  * (cs_ch_boundary), replays the two device phases on the host in the kernels' order of operations
  * for a fixed pseudo-random right-hand side b in [-1, 1), and writes the backward error
  * ||L x - b||_inf / ((1 + 16 a) ||x||_inf) of the result against the line operator L = I + a D4
- * itself.  CS_EINVAL for an invalid partition (n / chunks >= 16, a multiple of 8, chunks <= 64),
- * a < 0 or a non-finite a. */
+ * itself.  CS_EINVAL for an invalid partition (chunks <= 64 dividing n into n / chunks >= 16 points,
+ * a multiple of 8, or any length where n is a multiple of 64 and chunks a power of two), a < 0 or a
+ * non-finite a. */
 int cs_ch_solver_check(int64_t n, int32_t chunks, double a, int32_t boundary, double* residual);
 
 /* Allocation-free batched 1D sweep.  The paper has no counterpart: this entry point exists for

@@ -402,7 +402,8 @@ __device__ __forceinline__ void chain_lanes(const double* __restrict__ in, doubl
 
 // FP64 lines whose weights are c n_k with integers n_k, sum |n_k| <= 64, in 64-bit fixed point.  At two
 // FP64 instructions per clock and SM the five multiply-adds of a radius-2 stencil bound the FP64 walk at
-// 634 us for 63.5 M elements (FP32 storage 84 us; the floor of 16 bytes an element is 150 us).  Here a
+// 634 us for 63.5 M elements (FP32 storage 84 us; the floor of 16 bytes an element is 150 us), now 297 us, 122
+// instructions an element, bound by latency and the integer pipes (issue 67 %, ALU 53 %, FP64 42 %).  Here a
 // lane's window (8 elements and the neighbours that their stencils reach) becomes integers of 57 to 63 bits of
 // the window's largest value (63 with the bits that the sum takes), the weighted sums are exact, and the
 // one FP64 instruction left converts the scaled sum; what the weights miss of c n_k joins the sum as an

@@ -19,9 +19,9 @@
 // PENT): cs_penta.cuh's factored recursions in 64-bit fixed point, every line cut into P chunks of
 // m = n / P points, one thread per (line, chunk).  Two launches a step, one along the rows and one along
 // the columns with the update fused; each holds its lines in shared memory, so the field is read
-// once and written once.  4096^2, FP64 storage, periodic: rows 160 us (DRAM floor 39 us, bound by the
-// integer pipes at ~250 issue slots of a scheduler per 32 points), columns 223 us (floor 59 us), the step
-// 0.857 -> 0.582 ms; 1024^2 110 -> 63 us.
+// once and written once.  4096^2, FP64 storage, periodic: rows 166 us (DRAM floor 39 us, bound by the
+// integer pipes), columns 232 us (floor 59 us), the step
+// 0.60 ms (0.86 ms with FP64 recursions); 1024^2 65 us (110).
 //
 // No-flux boundaries (cs_ch_desc.boundary = CS_CH_NOFLUX): the same step on a cell-centred
 // grid whose stencils read ghost cells by even reflection.  Reflection commutes with the

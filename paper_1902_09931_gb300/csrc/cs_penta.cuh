@@ -2,7 +2,7 @@
 // difference's pentadiagonal system, in 64-bit fixed point on the integer pipe.
 //
 // GB300 issues FP64 at 1/64 of the FP32 rate, so an FP64 recursion of the minimal nine operations a
-// point is FP64-bound (the former solver took 0.64 of the 0.86 ms step at 4096^2).  A 64 x 64-bit
+// point is FP64-bound (0.64 ms for both directions at 4096^2; 0.40 ms in fixed point).  A 64 x 64-bit
 // fixed-point product is three 32 x 32 -> 64 multiply-adds, so the same recursion on the integer pipes
 // costs about a fifth of that, and it rounds at a fixed 2^-53 of the line chunk's largest right-hand
 // side or better, where FP64 rounds every partial sum (which grows to ~sqrt(a) times the
@@ -20,7 +20,7 @@
 //
 // Partition.  A line of n points is cut into P chunks of m.  Phase 1 runs both recursions on every
 // chunk from zero states and keeps four end values: the forward state (y, D) after the chunk and the
-// backward state (W, E = W_0 - W_1) before it.  The true states entering every chunk follow from
+// backward state (W, E = W_0 - W_1) before it, scaled by powers of two.  The true states entering every chunk follow from
 // these by 2 x 2 matrices (powers of the recursion's own matrix, a scan over the chunks; periodic
 // lines close through (I - M^P)^-1, reflected ones through the boundary's mirror conditions).  Phase 2
 // adds the four homogeneous responses to those states: x = W / c + sum of 4 table values times 4
@@ -28,11 +28,13 @@
 //
 // Fixed point.  b is scaled by its chunk's largest exponent so that |y|, |D| < 2^62 whatever the
 // data (the host sums the impulse responses' magnitudes); W likewise after a shift of y by s2 bits.
-// Chunks whose largest value is not finite or outside 2^[-900, 870] take the same recursion in FP64.
+// Chunks whose largest value is outside 2^[-900, 870] take the same recursion in FP64; a value that is not
+// finite fills its line with NaN.
 // All values live biased by 2^62 (unsigned), coefficients are 64-bit fractions split in 32-bit
 // words: a product is hi hi + (lo hi) / 2^32 + (hi lo) / 2^32, two taps share the three accumulators,
-// and the accumulators' initial values centre the rounding (the dropped lo lo term's mean included),
-// because a bias would be a drift of the conserved mass.  Zero data stay exactly zero: the
+// and the accumulators' initial values centre the rounding (the dropped lo lo term's mean included; b
+// itself is rounded to nearest), because a bias, or an error with the sign of a slowly varying field, would
+// be a drift of the conserved mass.  Zero data stay exactly zero: the
 // coefficients are multiples of 4, so the bias's own products are whole numbers.
 #pragma once
 
@@ -422,7 +424,7 @@ __host__ __device__ __forceinline__ double corr_native(const Par& q, int ew, uin
 }
 
 // ---- host: constants and tables --------------------------------------------------------------------
-// Double-double arithmetic (error-free sums and FMA products), ~2^-104.
+// Double-double arithmetic, ~2^-104: Knuth's two-sum, Dekker's renormalisation, products' errors by FMA.
 struct DD {
   double h, l;
   DD(double a = 0.0, double b = 0.0) : h(a), l(b) {}
